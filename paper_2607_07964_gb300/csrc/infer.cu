@@ -191,8 +191,6 @@ __device__ __forceinline__ void prefetch_l2(const void* src, uint32_t bytes) {
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Words a 32-bit word of codes is split into, one code per byte.
 template <int PB>
@@ -691,28 +689,6 @@ __global__ void __launch_bounds__((H28 ? 28 : 1) * (1 << LG) / 16) infer_out_reg
     }
 }
 
-// Launch as a programmatic dependent of the preceding work on the stream, in clusters of
-// `cluster` CTAs when cluster > 1.
-template <typename... Params, typename... Args>
-cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                             unsigned cluster, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = cluster;
-    at[1].val.clusterDim.y = 1;
-    at[1].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = cluster > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
-}
-
 // Shared-memory plan of the streaming kernel: x' (B d_in floats), then per slot the parked
 // lane sums (qps 4 S B floats, rounded to 16 bytes) and the stage's codes, scales and zeros.
 struct StreamPlan {
@@ -769,7 +745,7 @@ kq_status launch_out_reg(int64_t B, cudaStream_t st, const float* yp, int d_out,
                                      static_cast<int>(smem)));
         return KQ_OK;
     }));
-    KQ_CUDA(launch_dependent(infer_out_reg_kernel<LG, H28>, dim3(static_cast<unsigned>(B)), dim3(NT), smem, st, 1u, yp,
+    KQ_CUDA(launch_dependent(infer_out_reg_kernel<LG, H28>, dim3(static_cast<unsigned>(B)), dim3(NT), smem, st, 1u, true, yp,
                              d_out, s_g, su, y));
     KQ_LAUNCH_CHECK("infer_out_reg_kernel");
     return KQ_OK;
@@ -791,14 +767,14 @@ inline kq_status launch_out(int64_t B, cudaStream_t st, const float* yp, int d_o
     }
     if (h28o) {
         KQ_CUDA(launch_dependent(infer_out_kernel<7>, dim3(static_cast<unsigned>(7 * B)), dim3(256),
-                                 static_cast<size_t>(4) * (size_t{1} << lgo) * sizeof(float), st, 7u, yp, d_out, lgo, s_g,
+                                 static_cast<size_t>(4) * (size_t{1} << lgo) * sizeof(float), st, 7u, true, yp, d_out, lgo, s_g,
                                  su, y));
     } else if (d_out >= 64) {
         KQ_CUDA(launch_dependent(infer_out_kernel<8>, dim3(static_cast<unsigned>(8 * B)), dim3(256),
-                                 (size_t{1} << (lgo - 3)) * sizeof(float), st, 8u, yp, d_out, lgo - 3, s_g, su, y));
+                                 (size_t{1} << (lgo - 3)) * sizeof(float), st, 8u, true, yp, d_out, lgo - 3, s_g, su, y));
     } else {
         KQ_CUDA(launch_dependent(infer_out_kernel<1>, dim3(static_cast<unsigned>(B)), dim3(256),
-                                 static_cast<size_t>(d_out) * sizeof(float), st, 1u, yp, d_out, lgo, s_g, su, y));
+                                 static_cast<size_t>(d_out) * sizeof(float), st, 1u, true, yp, d_out, lgo, s_g, su, y));
     }
     KQ_LAUNCH_CHECK("infer_out_kernel");
     return KQ_OK;
@@ -815,7 +791,7 @@ kq_status launch_stream_b(const StreamPlan& sp, cudaStream_t st, const uint32_t*
                                      static_cast<int>(kStreamSmemMax)));
         return KQ_OK;
     }));
-    KQ_CUDA(launch_dependent(infer_stream_kernel<PB, B>, dim3(sp.grid), dim3(IS_WARPS * 32), sp.smem, st, 1u, packed, scale,
+    KQ_CUDA(launch_dependent(infer_stream_kernel<PB, B>, dim3(sp.grid), dim3(IS_WARPS * 32), sp.smem, st, 1u, true, packed, scale,
                              zero, d_out, d_in, ng, grouped, s_x, sv, lgi, h28i, x, yp, sp.qps, sp.nslot, sp.part_slot,
                              sp.slot_bytes, sp.xp, info));
     KQ_LAUNCH_CHECK("infer_stream_kernel");

@@ -77,6 +77,36 @@ struct SideStream {
 };
 SideStream* side_stream(cudaStream_t caller);
 
+// Launch in clusters of `cluster` CTAs (when > 1) and, with `dependent`, as a programmatic
+// dependent of the preceding kernel on the stream: it may start before that kernel has
+// finished, and touches what that kernel writes only after pdl_wait().
+template <typename... Params, typename... Args>
+cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                             unsigned cluster, bool dependent, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    unsigned n = 0;
+    if (dependent) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = cluster;
+        at[n].val.clusterDim.y = 1;
+        at[n++].val.clusterDim.z = 1;
+    }
+    cfg.attrs = at;
+    cfg.numAttrs = n;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+}
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------------ debug bounds checks
 // In the debug build (libkronq_debug.so, compiled with -DKQ_DEBUG), KQ_IN_RANGE(i, n) checks
 // 0 <= i < n for an index into a buffer of n elements before the kernel accesses it: a

@@ -17,8 +17,9 @@
 //             acc = fma(-wpre_k, P_kc, acc) over ascending k; w_c = w_c - acc
 // Kernels:
 //   rowgrid_kernel   per-row grid (group = 0) from the whole row before the sweep
-//   pack_r_kernel    the diagonal 128 x 128 blocks of R in the block kernel's layout
-//   obs_block_kernel 8 lanes per row, 16 columns per lane; the block's R in shared memory
+//   pack_r_kernel    the diagonal 128 x 128 blocks of R as the block kernel's 16 x 16 tiles
+//   pack_rq_kernel   the blocks of R right of them, for the fused update
+//   obs_block_kernel 32 rows per CTA, lane = row, 16 columns per warp
 //   trailing_kernel  128 x 128 output tiles of the shared tile GEMM (tile_gemm.cuh)
 //   colloss_kernel   col_loss[j] = sum over rows of E_j^2, fixed order (sumsq.cuh)
 #include <math.h>
@@ -87,472 +88,581 @@ __global__ void rowgrid_kernel(const float* __restrict__ W, int64_t d_out, int64
     }
 }
 
-// One block [i0, e) of the sweep for all rows. A group of LPR = 8 lanes handles one row;
-// lane position lp holds the CPL = 16 consecutive columns i0 + CPL lp + t of it in
-// registers. Column j = CPL o + jj is owned by lane o: for each o (rolled loop) the 16
-// columns are an unrolled loop, so every register index is a compile-time constant. Per
-// column the owner's w_j is broadcast in the group, every lane computes the (identical)
-// quantization and error, and every lane updates all CPL of its registers with R_jk. The
-// updates of columns k < j (lanes before the owner, or the owner's own earlier columns)
-// read R_jk = 0 or hit values that are no longer read, so no update needs a predicate and
-// the live columns k > j see exactly the operations of the definition.
-#ifndef KQ_OBS_LANES_PER_ROW
-#define KQ_OBS_LANES_PER_ROW 8
-#endif
-constexpr int LPR = KQ_OBS_LANES_PER_ROW;   // lanes per row (8 or 16)
-constexpr int CPL = BLK / LPR;              // columns per lane
-constexpr int NV = CPL / 4;                 // float4 slots per lane
-static_assert(LPR == 8 || LPR == 16, "lanes per row must be 8 or 16");
-// 32 rows per CTA (8 warps): with 64 KB of shared memory and at most 128 registers a
-// thread, a CTA fits beside one CTA of the 3xTF32 far-column update (129 KB, 320 threads),
-// so block b + 1 runs while block b's far columns are updated (one CTA per SM up to 4864
-// rows, two beyond).
+// One block [i0, e) of the sweep. A CTA takes 32 rows, lane = row, and its 8 warps take 16
+// consecutive columns each (warp s: columns i0 + 16 s ..), held in registers. The column loop
+// is a serial chain per row: quantize w_j, form E_j, update w_{j+1}. Warp o runs the chain of
+// its 16 columns with every value of a row in one lane (no exchange inside the 16 columns),
+// and after every 4 columns publishes their E (and with P the values before quantization)
+// through shared memory and one mbarrier arrival; the warps s > o, which own the later
+// columns, then apply those 4 columns' updates while warp o goes on, so that warp o + 1
+// starts its own chain a few fma after warp o's last column. Every column still receives
+// the updates j = 0, 1, ... in order with the definition's operations.
+// Bound: the chain's latency, ~20 dependent operations a column (two corrected divisions of 5,
+// rounding 2, clamp 2, product, difference, update): 140-165 cycles a column measured, plus
+// ~350-500 cycles for each of the seven hand-overs and ~5000 before the first column.
+// 4096 rows (128 CTAs): 30.3 k cycles, 14.6 us a block; the form with 8 lanes per row and a
+// shuffle per column took 25 us. With it the sweep of 1024 x 8192 went from 2.62 to 1.75 ms,
+// of 14336 x 4096 (three CTAs per SM) from 3.40 to 2.29 ms. A fully unrolled chain with one
+// register per column and range tests that branch took 270 cycles a column; packed pairs
+// (f32x2 fma) for the updates, 16 against 30 instructions, took 170 to 145.
+constexpr int CW = 16;                      // columns per warp
+constexpr int NWARP = BLK / CW;             // 8 warps
 constexpr int OBS_ROWS = 32;                // rows per CTA
-constexpr int OBS_THREADS = OBS_ROWS * LPR; // 256 or 512
-// With P the CTA holds both diagonal blocks (R and P, 128 KB): one CTA per SM, alone.
-constexpr int OBS_ROWS_P = 32;
-// Dynamic shared memory of the block kernel with the tensor-core fused update: R's block
-// and 32 rows of E_prev (padded), 80.5 KB -- still beside a 129 KB far-update CTA.
-constexpr int OBS_SMEM_MMA = (BLK * BLK + 32 * (BLK + 4)) * 4;
-constexpr int OBS_THREADS_P = OBS_ROWS_P * LPR;
+constexpr int OBS_THREADS = 32 * NWARP;
+constexpr int PUB = 4;                      // columns per publication
+constexpr int NPUB = BLK / PUB;             // publications (one mbarrier each)
+constexpr int ELD = OBS_ROWS + 2;           // column stride of the exchange tiles [16][ELD]: 8 rows x 4
+                                            // column quads of a transposing access hit 32 banks
+constexpr int XT = CW * ELD;                // floats of one warp's exchange tile
+constexpr int PLD = BLK + 4;                // row stride of the staged E_prev
+// Packed diagonal block of R: the 16 x 16 tiles (o, s), o <= s, the only ones the block's
+// column loop reads (36 of 64), tile s (s + 1) / 2 + o, row-major; the diagonal tiles (s, s)
+// with row jj shifted left by 4 (jj / 4): [jj][t] = R[jj][4 (jj / 4) + t] (0 past the tile). The
+// chain shifts its registers the same way after every 4 columns, so its loop has fixed
+// register indices and a body of 4 columns.
+constexpr int RT = CW * CW;
+constexpr int RTILES = NWARP * (NWARP + 1) / 2;
+constexpr int RPACK = RTILES * RT;          // 9216 floats, 36 KB
+__host__ __device__ constexpr int rtile(int o, int s) { return (s * (s + 1) / 2 + o) * RT; }
+// Shared memory: R's tiles (with P also P's), the exchange tiles of E (with P also of Wpre).
+// 54 KB (GPTQ mode): four CTAs per SM by shared memory, or one beside a 129 KB far-update CTA.
+constexpr int obs_smem(bool hasp) { return (hasp ? 2 : 1) * (RPACK + NWARP * XT) * static_cast<int>(sizeof(float)); }
+static_assert(OBS_ROWS * PLD <= NWARP * XT, "E_prev is staged in the exchange tiles");
+// How the previous block's lazy update of this block column is applied.
+enum { FUSE_NONE = 0, FUSE_FP32 = 1, FUSE_MMA = 2 };
 
-// Packed layout of one diagonal block of R: row j holds R[i0 + j][i0 + c] at pos(c). The
-// CPL columns of lane lp fill slots [lp NV, lp NV + NV) of 16 bytes, rotated by lane so
-// that the NV float4 loads of 8 consecutive lanes hit 8 distinct bank groups.
-__host__ __device__ constexpr int slot_of(int lp, int v) { return lp * NV + ((v + ((lp * NV) >> 3)) & (NV - 1)); }
-__device__ __forceinline__ int pos_of(int c) { return 4 * slot_of(c / CPL, (c % CPL) >> 2) + (c & 3); }
+// Rp[b][tile(o, s)][jj][t] = R[i0 + 16 o + jj][i0 + 16 s + t] = Lt[i0 + 16 s + t][i0 + 16 o + jj]
+// (0 outside the matrix; diagonal tiles shifted as above), i0 = b BLK. Grid (RTILES, blocks), block (16, 16): one tile.
+__global__ void pack_r_kernel(const float* __restrict__ Lt, int64_t n, float* __restrict__ Rp) {
+    __shared__ float t[CW][CW + 1];
+    int s = 0, o = static_cast<int>(blockIdx.x);
+    while (o > s) {
+        o -= s + 1;
+        ++s;
+    }
+    const int64_t i0 = static_cast<int64_t>(blockIdx.y) * BLK;
+    const int64_t c = i0 + CW * s + threadIdx.y, j = i0 + CW * o + threadIdx.x;
+    t[threadIdx.y][threadIdx.x] = (c < n && j < n) ? Lt[c * n + j] : 0.0f;
+    __syncthreads();
+    const int64_t e = static_cast<int64_t>(blockIdx.y) * RPACK + rtile(o, s) + threadIdx.y * CW + threadIdx.x;
+    const int jj = threadIdx.y;
+    int tt = threadIdx.x;   // column within the tile
+    if (o == s) tt += PUB * (jj / PUB);
+    if (KQ_IN_RANGE(e, static_cast<int64_t>(gridDim.y) * RPACK)) Rp[e] = tt < CW ? t[tt][jj] : 0.0f;
+}
 
-// Rp[b][j][pos(c)] = R[i0 + j][i1 + c] = Lt[i1 + c][i0 + j] (0 outside the matrix),
-// i0 = b BLK, i1 = i0 + coff BLK: the diagonal blocks (coff = 0) or the blocks right of them
-// (coff = 1). Block (32, 8) transposes one 32 x 32 tile through shared memory.
-__global__ void pack_r_kernel(const float* __restrict__ Lt, int64_t n, float* __restrict__ Rp, int coff) {
-    __shared__ float t[32][33];
-    const int64_t i0 = static_cast<int64_t>(blockIdx.z) * BLK;
-    const int64_t i1 = i0 + static_cast<int64_t>(coff) * BLK;
-    const int c0 = blockIdx.y * 32, j0 = blockIdx.x * 32;
-    for (int r = threadIdx.y; r < 32; r += 8) {
-        const int64_t c = i1 + c0 + r, j = i0 + j0 + threadIdx.x;
-        t[r][threadIdx.x] = (c < n && j < n) ? Lt[c * n + j] : 0.0f;
+// The block of R right of diagonal block b (rows i0 + k, columns i0 + BLK + c; 0 outside the
+// matrix) for the fused update. FRAG = false: Rq[b][s][k][t], c = 16 s + t: warp s reads a row
+// of 16 columns as four uniform 16-byte loads. FRAG = true: Rq[b][s][ks][lane][4] =
+// (R[8 ks + t4][c], R[8 ks + t4 + 4][c], the same at c + 8), c = 16 s + g, g = lane / 4,
+// t4 = lane % 4: the B fragments of mma.sync m16n8k8 for warp s's two column tiles, one
+// 16-byte load per lane and k step. Grid (8, blocks), block 256.
+template <bool FRAG>
+__global__ void pack_rq_kernel(const float* __restrict__ Lt, int64_t n, float* __restrict__ Rq) {
+    const int s = static_cast<int>(blockIdx.x);
+    const int64_t i0 = static_cast<int64_t>(blockIdx.y) * BLK, i1 = i0 + BLK + CW * s;
+    float* out = Rq + static_cast<int64_t>(blockIdx.y) * BLK * BLK + s * BLK * CW;
+    __shared__ float t[CW][BLK + 1];
+    for (int e = threadIdx.x; e < CW * BLK; e += blockDim.x) {
+        const int c = e / BLK, k = e % BLK;
+        t[c][k] = (i1 + c < n && i0 + k < n) ? Lt[(i1 + c) * n + i0 + k] : 0.0f;
     }
     __syncthreads();
-    float* out = Rp + static_cast<int64_t>(blockIdx.z) * BLK * BLK;
-    for (int r = threadIdx.y; r < 32; r += 8) {
-        const int j = j0 + r, c = c0 + threadIdx.x;
-        if (KQ_IN_RANGE(j * BLK + pos_of(c), BLK * BLK)) out[j * BLK + pos_of(c)] = t[threadIdx.x][r];
-    }
-}
-
-// Rq[b][c][k ^ (4 (c & 7))] = R[i0 + k][i1 + c] = Lt[i1 + c][i0 + k] (0 outside the matrix),
-// i0 = b BLK, i1 = i0 + BLK: the block of R right of diagonal block b, column-major with
-// the k index swizzled within 32-float groups, for the tensor-core form of the fused update
-// (its fragment loads then hit 32 banks). Block (32, 8), one 32 x 32 tile per CTA; Lt rows
-// are contiguous in k, so no transpose.
-__global__ void pack_rq_mma_kernel(const float* __restrict__ Lt, int64_t n, float* __restrict__ Rq) {
-    const int64_t i0 = static_cast<int64_t>(blockIdx.z) * BLK, i1 = i0 + BLK;
-    const int k0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-    float* out = Rq + static_cast<int64_t>(blockIdx.z) * BLK * BLK;
-    for (int r = threadIdx.y; r < 32; r += 8) {
-        const int c = c0 + r, k = k0 + threadIdx.x;
-        const int64_t lr = i1 + c, lc = i0 + k;
-        if (KQ_IN_RANGE(c * BLK + (k ^ (4 * (c & 7))), BLK * BLK))
-            out[c * BLK + (k ^ (4 * (c & 7)))] = (lr < n && lc < n) ? Lt[lr * n + lc] : 0.0f;
-    }
-}
-
-// The previous block's lazy update of this block column for the CTA's 32 rows on the tensor
-// cores (mma.sync m16n8k8 tf32, 3xTF32 split): C = E_prev R_prev,this with E_prev staged in
-// Es ([32][BLK + 4]) and R_prev,this in Rs (pack_rq_mma_kernel's layout); 8 warps of 16 x 32.
-// C is left in Es (same layout) after a barrier.
-__device__ __forceinline__ void prev_block_update_mma(float* Es, const float* Rs) {
-    constexpr int ESLD = BLK + 4;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, g = lane >> 2, t4 = lane & 3;
-    const int wr = wid >> 2, wc = wid & 3;
-    float c[4][4];
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) c[nt][e] = 0.0f;
-    const float* a0p = Es + (16 * wr + g) * ESLD;
-    const float* a1p = a0p + 8 * ESLD;
-#pragma unroll 2
-    for (int ks = 0; ks < BLK; ks += 8) {
-        const float a[4] = {a0p[ks + t4], a1p[ks + t4], a0p[ks + t4 + 4], a1p[ks + t4 + 4]};
-        uint32_t ah[4], al[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float hi = tf32_hi(a[e]);
-            ah[e] = __float_as_uint(hi);
-            al[e] = __float_as_uint(a[e] - hi);
+    for (int e = threadIdx.x; e < CW * BLK; e += blockDim.x) {
+        float v;
+        if constexpr (FRAG) {
+            const int u = e & 3, lane = (e >> 2) & 31, ks = e >> 7;
+            v = t[(lane >> 2) + 8 * (u >> 1)][8 * ks + (lane & 3) + 4 * (u & 1)];
+        } else {
+            v = t[e % CW][e / CW];
         }
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            const int col = 32 * wc + 8 * nt + g;   // col & 7 == g
-            const float b0 = Rs[col * BLK + ((ks + t4) ^ (4 * g))];
-            const float b1 = Rs[col * BLK + ((ks + t4 + 4) ^ (4 * g))];
-            const float bh0 = tf32_hi(b0), bh1 = tf32_hi(b1);
-            const uint32_t bh[2] = {__float_as_uint(bh0), __float_as_uint(bh1)};
-            const uint32_t bl[2] = {__float_as_uint(b0 - bh0), __float_as_uint(b1 - bh1)};
-            mma_tf32(c[nt], al, bh);
-            mma_tf32(c[nt], ah, bl);
-            mma_tf32(c[nt], ah, bh);
-        }
+        if (KQ_IN_RANGE(e, CW * BLK)) out[e] = v;
     }
-    __syncthreads();   // every warp is done with Es
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-        const int r = 16 * wr + g, col = 32 * wc + 8 * nt + 2 * t4;
-        Es[r * ESLD + col] = c[nt][0];
-        Es[r * ESLD + col + 1] = c[nt][1];
-        Es[(r + 8) * ESLD + col] = c[nt][2];
-        Es[(r + 8) * ESLD + col + 1] = c[nt][3];
-    }
-    __syncthreads();
 }
 
-__device__ __forceinline__ float group_min(float v) {
-    for (int o = LPR / 2; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-__device__ __forceinline__ float group_max(float v) {
-    for (int o = LPR / 2; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-
-// A lane's CPL columns [cb, cb + CPL) of row r of the block starting at column i0 (0 past
-// the block end nb or past the last row).
-// NC: through the read-only path (data this kernel does not write); else plain loads.
-template <bool VEC, bool NC = true>
-__device__ __forceinline__ void load_cols(const float* __restrict__ W, int64_t r, int64_t d_out, int64_t d_in,
-                                          int64_t i0, int cb, int nb, float (&w)[CPL]) {
-    const bool live = r < d_out;
-    const float* src = W + r * d_in + i0 + cb;
-    if (VEC && cb + CPL <= nb) {
+// Warp `warp`'s 16 columns of the CTA's rows in the transposing layout: lane (8 rows x 4 quads)
+// holds rows r0 + 8 it + lane / 4, columns c0 + 4 (lane % 4) .. + 3 of M (0 past row d_out or
+// column cend).
+template <bool VEC>
+__device__ __forceinline__ void load_quads(const float* M, int64_t r0, int64_t d_out, int64_t d_in,
+                                           int64_t c0, int64_t cend, float4 (&v)[4]) {
+    const int lane = threadIdx.x & 31;
+    const int64_t c = c0 + 4 * (lane & 3);
+    if (VEC && r0 + OBS_ROWS <= d_out && c0 + CW <= cend) {   // the whole tile
+        const float* p = M + (r0 + (lane >> 2)) * d_in + c;
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            const float4* p = reinterpret_cast<const float4*>(src) + v;
-            const float4 x = live ? (NC ? __ldg(p) : *p) : make_float4(0.f, 0.f, 0.f, 0.f);
-            w[4 * v] = x.x;
-            w[4 * v + 1] = x.y;
-            w[4 * v + 2] = x.z;
-            w[4 * v + 3] = x.w;
+        for (int it = 0; it < 4; ++it) v[it] = *reinterpret_cast<const float4*>(p + it * 8 * d_in);
+        return;
+    }
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+        const int64_t r = r0 + 8 * it + (lane >> 2);
+        v[it] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (r >= d_out) continue;
+        const float* p = M + r * d_in + c;
+        if (VEC && c + 3 < cend) {
+            v[it] = *reinterpret_cast<const float4*>(p);
+        } else {
+            if (c < cend) v[it].x = p[0];
+            if (c + 1 < cend) v[it].y = p[1];
+            if (c + 2 < cend) v[it].z = p[2];
+            if (c + 3 < cend) v[it].w = p[3];
         }
-    } else {
-#pragma unroll
-        for (int t = 0; t < CPL; ++t) w[t] = (live && cb + t < nb) ? src[t] : 0.0f;
     }
 }
 
 template <bool VEC>
-__device__ __forceinline__ void store_cols(float* W, int64_t r, int64_t d_out, int64_t d_in, int64_t i0, int cb,
-                                           int nb, const float (&w)[CPL]) {
-    if (r >= d_out || !KQ_IN_RANGE(r * d_in + i0 + cb + min(CPL, nb - cb) - 1, d_out * d_in)) return;
-    float* dst = W + r * d_in + i0 + cb;
-    if (VEC && cb + CPL <= nb) {
-#pragma unroll
-        for (int v = 0; v < NV; ++v)
-            reinterpret_cast<float4*>(dst)[v] = make_float4(w[4 * v], w[4 * v + 1], w[4 * v + 2], w[4 * v + 3]);
+__device__ __forceinline__ void store_quad(float* M, int64_t r, int64_t d_out, int64_t d_in, int64_t c, int64_t cend,
+                                           const float (&v)[4]) {
+    if (r >= d_out || c >= cend || !KQ_IN_RANGE(r * d_in + (c + 3 < cend ? c + 3 : cend - 1), d_out * d_in)) return;
+    float* p = M + r * d_in + c;
+    if (VEC && c + 3 < cend) {
+        *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
     } else {
 #pragma unroll
-        for (int t = 0; t < CPL; ++t)
-            if (cb + t < nb) dst[t] = w[t];
+        for (int u = 0; u < 4; ++u)
+            if (c + u < cend) p[u] = v[u];
     }
 }
 
-// w -= E_prev R_prev,this for one row: the previous block's lazy update of this block
-// column, in the order of the trailing update (acc = fma(E_k, R_kc, acc) over ascending k,
-// then w - acc). Rq: the block of R (rows = the previous block's columns) packed like the
-// diagonal blocks, in shared memory; ep: this lane's CPL entries of the row of E_prev.
-__device__ __forceinline__ void prev_block_update(const float* Rq, const float (&ep)[CPL], int lp, int gbase,
-                                                  float (&w)[CPL]) {
-    float acc[CPL];
+// The previous block's lazy update of warp s's 16 columns for the CTA's 32 rows on the tensor
+// cores (mma.sync m16n8k8 tf32, 3xTF32 split, ascending k): C = E_prev R_prev,this with E_prev
+// staged in Es ([32][PLD]) and the lane's B fragments of every k step in registers (each CTA
+// reads every fragment once). c[mt][nt]: rows 16 mt, columns 8 nt of the warp's 32 x 16 tile.
+__device__ __forceinline__ void prev_block_update_mma(const float* Es, const float4 (&frag)[BLK / 8], float (&c)[2][2][4]) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
 #pragma unroll
-    for (int t = 0; t < CPL; ++t) acc[t] = 0.0f;
-#pragma unroll 1
-    for (int o = 0; o < LPR; ++o) {
+    for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-        for (int jj = 0; jj < CPL; ++jj) {
-            const float ek = __shfl_sync(0xffffffffu, ep[jj], gbase | o);
-            const float* rr = Rq + (CPL * o + jj) * BLK;
+        for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                const float4 x = *reinterpret_cast<const float4*>(rr + 4 * slot_of(lp, v));
-                acc[4 * v] = __fmaf_rn(ek, x.x, acc[4 * v]);
-                acc[4 * v + 1] = __fmaf_rn(ek, x.y, acc[4 * v + 1]);
-                acc[4 * v + 2] = __fmaf_rn(ek, x.z, acc[4 * v + 2]);
-                acc[4 * v + 3] = __fmaf_rn(ek, x.w, acc[4 * v + 3]);
+            for (int e = 0; e < 4; ++e) c[mt][nt][e] = 0.0f;
+#pragma unroll
+    for (int ks = 0; ks < BLK / 8; ++ks) {
+        const float4 bf = frag[ks];
+        const float b[2][2] = {{bf.x, bf.y}, {bf.z, bf.w}};
+        uint32_t bh[2][2], bl[2][2];
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float hi = tf32_hi(b[nt][e]);
+                bh[nt][e] = __float_as_uint(hi);
+                bl[nt][e] = __float_as_uint(b[nt][e] - hi);
+            }
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) {
+            const float* a0p = Es + (16 * mt + g) * PLD + 8 * ks;
+            const float* a1p = a0p + 8 * PLD;
+            const float a[4] = {a0p[t4], a1p[t4], a0p[t4 + 4], a1p[t4 + 4]};
+            uint32_t ah[4], al[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float hi = tf32_hi(a[e]);
+                ah[e] = __float_as_uint(hi);
+                al[e] = __float_as_uint(a[e] - hi);
+            }
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt) {
+                mma_tf32(c[mt][nt], al, bh[nt]);
+                mma_tf32(c[mt][nt], ah, bl[nt]);
+                mma_tf32(c[mt][nt], ah, bh[nt]);
             }
         }
     }
-#pragma unroll
-    for (int t = 0; t < CPL; ++t) w[t] = __fsub_rn(w[t], acc[t]);
 }
 
-// VEC: d_in % 16 == 0 and W, codes (and pre_q) 16-byte aligned, so a lane's CPL columns
-// of W, E and codes move as 16-byte vectors. HASP: with the GPTAQ correction; Pp is P's
+// The same in fp32 in the order of the trailing update (acc = fma(E_k, R_kc, acc) over
+// ascending k) for the lane's row; rq: warp s's columns of R_prev,this ([BLK][16]).
+__device__ __forceinline__ void prev_block_update(const float* Es, const float* __restrict__ rq, float (&acc)[CW]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int t = 0; t < CW; ++t) acc[t] = 0.0f;
+#pragma unroll 2
+    for (int k = 0; k < BLK; k += 4) {
+        const float4 e4 = *reinterpret_cast<const float4*>(Es + lane * PLD + k);
+        const float ek[4] = {e4.x, e4.y, e4.z, e4.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const float4* rr = reinterpret_cast<const float4*>(rq + (k + u) * CW);
+#pragma unroll
+            for (int v = 0; v < CW / 4; ++v) {
+                const float4 x = __ldg(rr + v);
+                acc[4 * v] = __fmaf_rn(ek[u], x.x, acc[4 * v]);
+                acc[4 * v + 1] = __fmaf_rn(ek[u], x.y, acc[4 * v + 1]);
+                acc[4 * v + 2] = __fmaf_rn(ek[u], x.z, acc[4 * v + 2]);
+                acc[4 * v + 3] = __fmaf_rn(ek[u], x.w, acc[4 * v + 3]);
+            }
+        }
+    }
+}
+
+// One row's grid and the constants of its column steps: the integer t = q - zero is
+// rint(w / scale) clamped to [lo, hi] (the same number as clamp(rint + zero, 0, maxq) - zero:
+// all are integers below 2^24 or clamped alike).
+struct RowGrid {
+    float scale, ys, zero, lo, hi;
+};
+
+// What the column steps of a publication met: ok() when div_rn_fast was exact in all of them
+// (reciprocals aside). A quotient w / scale only has to round to the right integer: below 1/4
+// any error is harmless and above it the residuals are exact for every w, so w needs no lower
+// bound; the dividend of E must be 0 or at least 2^-60. nan collects 0 * w.
+struct StepRange {
+    float mx = 0.0f, mn = 1.0f, nan = 0.0f;
+    __device__ __forceinline__ bool ok() const { return (mx <= 0x1p60f) & (mn >= 0x1p-60f) & (nan == 0.0f); }
+};
+
+// One column step: t and E for the value w (d.x = 1 / R_jj, d.y = R_jj). !EXACT: div_rn_fast's
+// operations, written out; the sign of a zero quotient does not matter to the rounding of the
+// first division, which skips the a == 0 case; rounding is the addition of 1.5 * 2^23 (to
+// nearest even below 2^22; beyond, the clamp decides).
+template <bool EXACT>
+__device__ __forceinline__ void column_step(float w, const RowGrid& g, float2 d, float& t, float& err, StepRange& sr) {
+    if constexpr (EXACT) {
+        t = fminf(fmaxf(rintf(__fdiv_rn(w, g.scale)), g.lo), g.hi);
+        err = __fdiv_rn(__fsub_rn(w, __fmul_rn(g.scale, t)), d.y);
+    } else {
+        const float q0 = __fmul_rn(w, g.ys);
+        const float q1 = __fmaf_rn(__fmaf_rn(-q0, g.scale, w), g.ys, q0);
+        const float q2 = __fmaf_rn(__fmaf_rn(-q1, g.scale, w), g.ys, q1);
+        t = fminf(fmaxf(__fsub_rn(__fadd_rn(q2, 12582912.0f), 12582912.0f), g.lo), g.hi);
+        const float dif = __fsub_rn(w, __fmul_rn(g.scale, t));
+        err = div_rn_fast(dif, d.y, d.x);
+        sr.mx = fmaxf(sr.mx, fmaxf(fabsf(w), fabsf(dif)));
+        sr.mn = fminf(sr.mn, dif == 0.0f ? 1.0f : fabsf(dif));
+        sr.nan = __fmaf_rn(w, 0.0f, sr.nan);
+    }
+}
+
+// VEC: d_in % 16 == 0 and W, codes (and pre_q) 16-byte aligned, so a lane's columns of W, E
+// and codes move as 16-byte vectors. HASP: with the GPTAQ correction; Pp is P's
 // diagonal block packed like R's, and the block's -Wpre goes to Q (fp32 trailing update)
-// or to Qh + Ql (tensor-core trailing update).
-template <bool VEC, bool HASP>
-__global__ void __launch_bounds__(HASP ? OBS_THREADS_P : OBS_THREADS, HASP ? 1 : 2) obs_block_kernel(
-    float* __restrict__ W, int64_t d_out, int64_t d_in, const float* __restrict__ Rp, int64_t i0,
+// or to Qh + Ql (tensor-core trailing update). FUSE: the previous block's update of this
+// block column first (Rq: pack_rq_kernel's layout for that form). One CTA per 32 rows.
+template <bool VEC, bool HASP, int FUSE, int PER_SM = 2>
+__global__ void __launch_bounds__(OBS_THREADS, PER_SM) obs_block_kernel(
+    const float* W, int64_t d_out, int64_t d_in, const float* __restrict__ Rp, int64_t i0,
     int bits, int group, const float* __restrict__ gscale, const float* __restrict__ gzero,
     uint8_t* __restrict__ codes, float* __restrict__ scale, int32_t* __restrict__ zero,
-    float* __restrict__ E, float* __restrict__ pre_q, float* __restrict__ Eh, float* __restrict__ El,
+    float* E, float* __restrict__ pre_q, float* __restrict__ Eh, float* __restrict__ El,
     const float* __restrict__ Pp, float* __restrict__ Q, float* __restrict__ Qh, float* __restrict__ Ql,
-    const float* __restrict__ Rq, int fused_mma, int* info) {
-    extern __shared__ __align__(16) float Rs[];   // [BLK][BLK], packed (pack_r_kernel); then P's
-    float* Ps = Rs + BLK * BLK;
-    const bool fused = !HASP && Rq != nullptr;
-    // With Rq, the buffer first holds the previous block's R_prev,this for the fused update.
-    for (int e = threadIdx.x; e < BLK * BLK / 4; e += blockDim.x) cp_async16(Rs + 4 * e, (fused ? Rq : Rp) + 4 * e, 16);
-    if (HASP)
-        for (int e = threadIdx.x; e < BLK * BLK / 4; e += blockDim.x) cp_async16(Ps + 4 * e, Pp + 4 * e, 16);
-    cp_async_commit();
+    const float* __restrict__ Rq, int* info) {
+    extern __shared__ __align__(16) float Rs[];   // R's tiles, exchange tiles, with P: P's tiles, Wpre's exchange tiles
+    float* Xs = Rs + RPACK;
+    float* Ps = Xs + NWARP * XT;
+    float* Qs = Ps + RPACK;
+    __shared__ uint64_t pub[NPUB];
+    __shared__ float mnmx[2][NWARP][OBS_ROWS];
+    __shared__ float2 rds[BLK];
+    __shared__ int abort_flag, ieee_only;
+    const int lane = threadIdx.x & 31, s = threadIdx.x >> 5;
     const int nb = static_cast<int>(min(static_cast<int64_t>(BLK), d_in - i0));
-    const float maxq = static_cast<float>((1 << bits) - 1);
-    const int lane = threadIdx.x & 31;
-    const int lp = lane & (LPR - 1);
-    const int gbase = lane & ~(LPR - 1);
-    const int cb = CPL * lp;                       // first column of this lane in the block
-    const int64_t ngroups = group ? (d_in + group - 1) / group : 1;
-    const int warps = blockDim.x / 32;
-    constexpr int RPW = 32 / LPR;                  // rows per warp
-    const int64_t rstride = static_cast<int64_t>(gridDim.x) * warps * RPW;
-    const int64_t rw0 = (static_cast<int64_t>(blockIdx.x) * warps + threadIdx.x / 32) * RPW;
-    float w[CPL];
-    if (fused) {
-        // Each row of this CTA goes back to W updated, and the sweep below reads it with
-        // plain loads; then the diagonal block replaces R_prev,this in shared memory.
+    const int64_t row0 = static_cast<int64_t>(blockIdx.x) * OBS_ROWS;
+    const int64_t r = row0 + lane;
+    const bool live = r < d_out;
+    const int64_t cend = i0 + nb, c0 = i0 + CW * s;
+    if (threadIdx.x == 0) {
+        for (int k = 0; k < NPUB; ++k) mbar_init(&pub[k], 1);
+        fence_mbar_init();
+        abort_flag = 0;
+        ieee_only = 0;
+    }
+    // R (and P) do not depend on the kernel before this one (see block_launch): ahead of the wait
+    for (int e = threadIdx.x; e < RPACK / 4; e += OBS_THREADS) cp_async16(Rs + 4 * e, Rp + 4 * e, 16);
+    if constexpr (HASP)
+        for (int e = threadIdx.x; e < RPACK / 4; e += OBS_THREADS) cp_async16(Ps + 4 * e, Pp + 4 * e, 16);
+    cp_async_commit();
+    float4 frag[FUSE == FUSE_MMA ? BLK / 8 : 1];
+    if constexpr (FUSE == FUSE_MMA) {
+#pragma unroll
+        for (int ks = 0; ks < BLK / 8; ++ks) frag[ks] = __ldg(reinterpret_cast<const float4*>(Rq + s * BLK * CW) + 32 * ks + lane);
+    }
+    pdl_wait();
+    if constexpr (FUSE != FUSE_NONE) {   // E_prev (128 columns) of the CTA's rows into the exchange tiles
+        for (int q = threadIdx.x; q < OBS_ROWS * (BLK / 4); q += OBS_THREADS) {
+            const int rr = q / (BLK / 4), c4 = 4 * (q % (BLK / 4));
+            const bool lv = row0 + rr < d_out;
+            const float* src = E + (row0 + rr) * d_in + (i0 - BLK) + c4;
+            if constexpr (VEC) {
+                cp_async16(Xs + rr * PLD + c4, lv ? src : E, lv ? 16 : 0);
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) Xs[rr * PLD + c4 + u] = lv ? src[u] : 0.0f;
+            }
+        }
+        cp_async_commit();
+    }
+    float4 wq4[4];
+    load_quads<VEC>(W, row0, d_out, d_in, c0, cend, wq4);
+    float* xt = Xs + s * XT;                     // this warp's exchange tile
+    const int qr = lane >> 2, qc = 4 * (lane & 3);   // this lane's place in the transposing layout
+    float2 w[CW / 2];   // the warp's 16 columns of the lane's row, in pairs
+    if constexpr (FUSE == FUSE_MMA) {
         cp_async_wait<0>();
         __syncthreads();
-        if (VEC && fused_mma && rstride >= d_out) {
-            // tensor-core form (one row group per CTA: its 32 rows from blockIdx.x * 32)
-            constexpr int ESLD = BLK + 4;
-            float* Es = Rs + BLK * BLK;
-            const int64_t row0 = static_cast<int64_t>(blockIdx.x) * warps * RPW;
-            for (int q = threadIdx.x; q < 32 * (BLK / 4); q += blockDim.x) {
-                const int rr = q / (BLK / 4), c4 = q % (BLK / 4);
-                const bool lv = row0 + rr < d_out;
-                cp_async16(Es + rr * ESLD + 4 * c4, lv ? E + (row0 + rr) * d_in + (i0 - BLK) + 4 * c4 : E, lv ? 16 : 0);
+        float c[2][2][4];
+        prev_block_update_mma(Xs, frag, c);
+        __syncthreads();   // every warp is done with E_prev
+        const int g = lane >> 2, t2 = 2 * (lane & 3);
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt) {
+                float* x = xt + (8 * nt + t2) * ELD + 16 * mt + g;
+                x[0] = c[mt][nt][0];
+                x[ELD] = c[mt][nt][1];
+                x[8] = c[mt][nt][2];
+                x[ELD + 8] = c[mt][nt][3];
             }
-            cp_async_commit();
+        __syncwarp();
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {   // W - C in place: each lane its own elements
+            float* x = xt + qc * ELD + 8 * it + qr;
+            x[0] = __fsub_rn(wq4[it].x, x[0]);
+            x[ELD] = __fsub_rn(wq4[it].y, x[ELD]);
+            x[2 * ELD] = __fsub_rn(wq4[it].z, x[2 * ELD]);
+            x[3 * ELD] = __fsub_rn(wq4[it].w, x[3 * ELD]);
+        }
+    } else {
+        float acc[CW];
+        if constexpr (FUSE == FUSE_FP32) {
             cp_async_wait<0>();
             __syncthreads();
-            prev_block_update_mma(Es, Rs);
-            const int64_t r = rw0 + lane / LPR;
-            const float* cu = Es + (r - row0) * ESLD + cb;
-            load_cols<VEC>(W, r, d_out, d_in, i0, cb, nb, w);
-#pragma unroll
-            for (int t = 0; t < CPL; ++t) w[t] = __fsub_rn(w[t], cu[t]);
-            store_cols<VEC>(W, r, d_out, d_in, i0, cb, nb, w);
-        } else {
-            for (int64_t rw = rw0; rw < d_out; rw += rstride) {
-                const int64_t r = rw + lane / LPR;
-                float ep[CPL];
-                load_cols<VEC>(E, r, d_out, d_in, i0 - BLK, cb, BLK, ep);
-                load_cols<VEC>(W, r, d_out, d_in, i0, cb, nb, w);
-                prev_block_update(Rs, ep, lp, gbase, w);
-                store_cols<VEC>(W, r, d_out, d_in, i0, cb, nb, w);
-            }
+            prev_block_update(Xs, Rq + s * BLK * CW, acc);
+            __syncthreads();   // every warp is done with E_prev
         }
-        __syncthreads();
-        for (int e = threadIdx.x; e < BLK * BLK / 4; e += blockDim.x) cp_async16(Rs + 4 * e, Rp + 4 * e, 16);
-        cp_async_commit();
-        load_cols<VEC, false>(W, rw0 + lane / LPR, d_out, d_in, i0, cb, nb, w);
-    } else {
-        // The first row's weights load while R is staged.
-        load_cols<VEC>(W, rw0 + lane / LPR, d_out, d_in, i0, cb, nb, w);
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+            float* x = xt + qc * ELD + 8 * it + qr;
+            x[0] = wq4[it].x;
+            x[ELD] = wq4[it].y;
+            x[2 * ELD] = wq4[it].z;
+            x[3 * ELD] = wq4[it].w;
+        }
+        if constexpr (FUSE == FUSE_FP32) {
+            __syncwarp();
+#pragma unroll
+            for (int t = 0; t < CW; ++t) xt[t * ELD + lane] = __fsub_rn(xt[t * ELD + lane], acc[t]);
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < CW / 2; ++t) w[t] = make_float2(xt[2 * t * ELD + lane], xt[(2 * t + 1) * ELD + lane]);
+    // The grid of the row: the minimum and maximum of the whole block (values past the end are 0,
+    // which the definition includes anyway).
+    if (group) {
+        float mn = 0.0f, mx = 0.0f;
+#pragma unroll
+        for (int t = 0; t < CW / 2; ++t) {
+            mn = fminf(mn, fminf(w[t].x, w[t].y));
+            mx = fmaxf(mx, fmaxf(w[t].x, w[t].y));
+        }
+        mnmx[0][s][lane] = mn;
+        mnmx[1][s][lane] = mx;
     }
     cp_async_wait<0>();
-    __syncthreads();   // every thread reaches it
-    // Reciprocals of the block's diagonal R_jj for the column steps' divisions.
-    __shared__ float rds[BLK];
-    for (int j = threadIdx.x; j < BLK; j += blockDim.x) rds[j] = j < nb ? div_recip(Rs[j * BLK + pos_of(j)]) : 0.0f;
     __syncthreads();
-    for (int64_t rw = rw0; rw < d_out; rw += rstride) {
-        const int64_t r = rw + lane / LPR;
-        const bool live = r < d_out;
-        if (rw != rw0) {
-            if (fused)
-                load_cols<VEC, false>(W, r, d_out, d_in, i0, cb, nb, w);
-            else
-                load_cols<VEC>(W, r, d_out, d_in, i0, cb, nb, w);
-        }
-        Grid g;
-        if (group) {
-            float mn = 0.0f, mx = 0.0f;
+    if (threadIdx.x < BLK) {   // reciprocals of the block's diagonal R_jj for the divisions
+        const int j = threadIdx.x;
+        // (columns past the end: finite steps, nothing kept)
+        const float dj = j < nb ? Rs[rtile(j / CW, j / CW) + (j % CW) * CW + j % PUB] : 1.0f;
+        const float y = div_recip(dj);
+        rds[j] = make_float2(y, dj);
+        if (y == 0.0f) ieee_only = 1;
+    }
+    const float maxq = static_cast<float>((1 << bits) - 1);
+    RowGrid g;
+    if (group) {
+        float mn = mnmx[0][0][lane], mx = mnmx[1][0][lane];
 #pragma unroll
-            for (int t = 0; t < CPL; ++t)
-                if (cb + t < nb) {
-                    mn = fminf(mn, w[t]);
-                    mx = fmaxf(mx, w[t]);
-                }
-            g = make_grid(group_min(mn), group_max(mx), maxq);
-            if (live && lp == 0 && KQ_IN_RANGE(r * ngroups + i0 / group, d_out * ngroups)) {
-                const int64_t gi = r * ngroups + i0 / group;
-                scale[gi] = g.scale;
-                zero[gi] = static_cast<int32_t>(g.zero);
-            }
-        } else {
-            g.scale = live ? gscale[r] : 1.0f;
-            g.zero = live ? gzero[r] : 0.0f;
+        for (int k = 1; k < NWARP; ++k) {
+            mn = fminf(mn, mnmx[0][k][lane]);
+            mx = fmaxf(mx, mnmx[1][k][lane]);
         }
-        const float ys = div_recip(g.scale);
-        bool finite = true;   // every value quantized in this row group was finite
-        // The column steps of this row group; EXACT: IEEE divisions, else div_rn_fast, with
-        // the return value telling whether every operand was inside its exact range.
-        auto sweep = [&](auto exact_tag) -> bool {
-        constexpr bool EXACT = decltype(exact_tag)::value;
-        bool ok = true;
+        const Grid gr = make_grid(mn, mx, maxq);
+        g.scale = gr.scale;
+        g.zero = gr.zero;
+        const int64_t ngroups = (d_in + BLK - 1) / BLK, gi = r * ngroups + i0 / BLK;   // group == BLK
+        if (live && s == 0 && KQ_IN_RANGE(gi, d_out * ngroups)) {
+            scale[gi] = g.scale;
+            zero[gi] = static_cast<int32_t>(g.zero);
+        }
+    } else {
+        g.scale = live ? gscale[r] : 1.0f;
+        g.zero = live ? gzero[r] : 0.0f;
+    }
+    g.ys = div_recip(g.scale);
+    g.lo = __fsub_rn(0.0f, g.zero);
+    g.hi = __fsub_rn(maxq, g.zero);
+    __syncthreads();
+    if (CW * s >= nb) return;   // no columns (a last block narrower than 128)
+    // The earlier warps' columns.
+    for (int o = 0; o < s; ++o) {
+        const float* rt = Rs + rtile(o, s);
+        const float* ex = Xs + o * XT;
 #pragma unroll 1
-        for (int o = 0; o < LPR; ++o) {
-            if (CPL * o >= nb) break;   // uniform across the CTA
-            float e[CPL];
-            float wq[HASP ? CPL : 1];   // the values before quantization (with P only)
-            (void)wq;
-            uint32_t cq[NV];
+        for (int p = 0; p < CW / PUB; ++p) {
+            if (!mbar_wait(&pub[o * (CW / PUB) + p], 0, &abort_flag)) {
+                if (lane == 0) record_error(info, -KQ_ERR_TIMEOUT);
+                return;
+            }
 #pragma unroll
-            for (int v = 0; v < NV; ++v) cq[v] = 0u;
+            for (int u = 0; u < PUB; ++u) {
+                const int jj = PUB * p + u;
+                const float ne = -ex[jj * ELD + lane];
+                const float2 ne2 = make_float2(ne, ne);
+                const float4* rr = reinterpret_cast<const float4*>(rt + jj * CW);
+                float2 wp2 = make_float2(0.0f, 0.0f);
+                if constexpr (HASP) wp2.x = wp2.y = Qs[o * XT + jj * ELD + lane];
+                (void)wp2;
 #pragma unroll
-            for (int jj = 0; jj < CPL; ++jj) {
-                const int j = CPL * o + jj;
-                e[jj] = 0.0f;
-                if (j < nb) {   // uniform across the CTA
-                    const float* rr = Rs + j * BLK;
-                    const float dj = rr[4 * slot_of(o, jj >> 2) + (jj & 3)];
-                    const float yd = rds[j];
-                    float4 rv[NV];
-#pragma unroll
-                    for (int v = 0; v < NV; ++v) rv[v] = *reinterpret_cast<const float4*>(rr + 4 * slot_of(lp, v));
-                    const float wj = __shfl_sync(0xffffffffu, w[jj], gbase | o);
-                    finite = finite & (fabsf(wj) <= 3.402823466e38f);
-                    float q0;
-                    if constexpr (EXACT) {
-                        q0 = __fdiv_rn(wj, g.scale);
-                    } else {
-                        q0 = div_rn_fast(wj, g.scale, ys);
-                        ok = ok & div_rn_fast_ok(wj, ys);
-                    }
-                    float qq = __fadd_rn(rintf(q0), g.zero);
-                    qq = fminf(fmaxf(qq, 0.0f), maxq);
-                    const float what = __fmul_rn(g.scale, __fsub_rn(qq, g.zero));
-                    const float dif = __fsub_rn(wj, what);
-                    float err;
-                    if constexpr (EXACT) {
-                        err = __fdiv_rn(dif, dj);
-                    } else {
-                        err = div_rn_fast(dif, dj, yd);
-                        ok = ok & div_rn_fast_ok(dif, yd);
-                    }
-                    e[jj] = err;
-                    cq[jj >> 2] |= static_cast<uint32_t>(qq) << (8 * (jj & 3));
-                    if (pre_q && live && lp == o && KQ_IN_RANGE(r * d_in + i0 + j, d_out * d_in))
-                        pre_q[r * d_in + i0 + j] = wj;
+                for (int v = 0; v < CW / 4; ++v) {
+                    const float4 x = rr[v];
+                    w[2 * v] = __ffma2_rn(ne2, make_float2(x.x, x.y), w[2 * v]);
+                    w[2 * v + 1] = __ffma2_rn(ne2, make_float2(x.z, x.w), w[2 * v + 1]);
                     if constexpr (HASP) {
-                        wq[jj] = wj;
-                        const float* pr = Ps + j * BLK;
-                        float4 pv[NV];
-#pragma unroll
-                        for (int v = 0; v < NV; ++v) pv[v] = *reinterpret_cast<const float4*>(pr + 4 * slot_of(lp, v));
-#pragma unroll
-                        for (int v = 0; v < NV; ++v) {
-                            w[4 * v] = __fmaf_rn(wj, pv[v].x, __fmaf_rn(-err, rv[v].x, w[4 * v]));
-                            w[4 * v + 1] = __fmaf_rn(wj, pv[v].y, __fmaf_rn(-err, rv[v].y, w[4 * v + 1]));
-                            w[4 * v + 2] = __fmaf_rn(wj, pv[v].z, __fmaf_rn(-err, rv[v].z, w[4 * v + 2]));
-                            w[4 * v + 3] = __fmaf_rn(wj, pv[v].w, __fmaf_rn(-err, rv[v].w, w[4 * v + 3]));
-                        }
-                    } else {
-#pragma unroll
-                        for (int v = 0; v < NV; ++v) {
-                            w[4 * v] = __fmaf_rn(-err, rv[v].x, w[4 * v]);
-                            w[4 * v + 1] = __fmaf_rn(-err, rv[v].y, w[4 * v + 1]);
-                            w[4 * v + 2] = __fmaf_rn(-err, rv[v].z, w[4 * v + 2]);
-                            w[4 * v + 3] = __fmaf_rn(-err, rv[v].w, w[4 * v + 3]);
-                        }
+                        const float4 y = reinterpret_cast<const float4*>(Ps + rtile(o, s) + jj * CW)[v];
+                        w[2 * v] = __ffma2_rn(wp2, make_float2(y.x, y.y), w[2 * v]);
+                        w[2 * v + 1] = __ffma2_rn(wp2, make_float2(y.z, y.w), w[2 * v + 1]);
                     }
-                } else if constexpr (HASP) {
-                    wq[jj] = 0.0f;
-                }
-            }
-            if (live && lp == o && KQ_IN_RANGE(r * d_in + i0 + min(CPL * o + CPL, nb) - 1, d_out * d_in)) {
-                const int64_t ob = r * d_in + i0 + CPL * o;
-                if (VEC && CPL * o + CPL <= nb) {
-#pragma unroll
-                    for (int v = 0; v < NV; ++v)
-                        reinterpret_cast<float4*>(E + ob)[v] = make_float4(e[4 * v], e[4 * v + 1], e[4 * v + 2], e[4 * v + 3]);
-                    if constexpr (NV == 4) {
-                        *reinterpret_cast<uint4*>(codes + ob) = make_uint4(cq[0], cq[1], cq[2], cq[3]);
-                    } else {
-                        *reinterpret_cast<uint2*>(codes + ob) = make_uint2(cq[0], cq[1]);
-                    }
-                    if (Eh) {   // tensor-core trailing update: E = E_hi + E_lo
-#pragma unroll
-                        for (int v = 0; v < NV; ++v) {
-                            float h[4], l[4];
-#pragma unroll
-                            for (int t = 0; t < 4; ++t) {
-                                h[t] = tf32_hi(e[4 * v + t]);
-                                l[t] = e[4 * v + t] - h[t];
-                            }
-                            reinterpret_cast<float4*>(Eh + ob)[v] = make_float4(h[0], h[1], h[2], h[3]);
-                            reinterpret_cast<float4*>(El + ob)[v] = make_float4(l[0], l[1], l[2], l[3]);
-                        }
-                    }
-                    if constexpr (HASP) {   // -Wpre of the block, for the trailing update
-                        if (Qh) {
-#pragma unroll
-                            for (int v = 0; v < NV; ++v) {
-                                float h[4], l[4];
-#pragma unroll
-                                for (int t = 0; t < 4; ++t) {
-                                    h[t] = tf32_hi(-wq[4 * v + t]);
-                                    l[t] = -wq[4 * v + t] - h[t];
-                                }
-                                reinterpret_cast<float4*>(Qh + ob)[v] = make_float4(h[0], h[1], h[2], h[3]);
-                                reinterpret_cast<float4*>(Ql + ob)[v] = make_float4(l[0], l[1], l[2], l[3]);
-                            }
-                        } else {
-#pragma unroll
-                            for (int v = 0; v < NV; ++v)
-                                reinterpret_cast<float4*>(Q + ob)[v] =
-                                    make_float4(-wq[4 * v], -wq[4 * v + 1], -wq[4 * v + 2], -wq[4 * v + 3]);
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int t = 0; t < CPL; ++t)
-                        if (CPL * o + t < nb) {
-                            E[ob + t] = e[t];
-                            codes[ob + t] = static_cast<uint8_t>(cq[t >> 2] >> (8 * (t & 3)));
-                            if (Eh) {
-                                const float h = tf32_hi(e[t]);
-                                Eh[ob + t] = h;
-                                El[ob + t] = e[t] - h;
-                            }
-                            if constexpr (HASP) {
-                                if (Qh) {
-                                    const float h = tf32_hi(-wq[t]);
-                                    Qh[ob + t] = h;
-                                    Ql[ob + t] = -wq[t] - h;
-                                } else {
-                                    Q[ob + t] = -wq[t];
-                                }
-                            }
-                        }
                 }
             }
         }
-        return ok;
-        };
-        if (!__all_sync(0xffffffffu, sweep(std::false_type{}))) {
-            // an operand outside the fast division's range in this warp's rows: the row
-            // group again from its start, with IEEE divisions (same outputs overwritten)
-            if (fused)
-                load_cols<VEC, false>(W, r, d_out, d_in, i0, cb, nb, w);
-            else
-                load_cols<VEC>(W, r, d_out, d_in, i0, cb, nb, w);
-            sweep(std::true_type{});
+    }
+    if (CW * (s + 1) >= nb) pdl_launch_dependents();   // the last warp: an eighth of the chain to go
+    // This warp's chain, 4 columns (w[0], w[1]) per turn of the loop, the last of which moves the
+    // later columns down by 4; the first 8 columns update 16 registers, the last 8 only 8.
+    const float* rt = Rs + rtile(s, s);
+    const float* pt = Ps + rtile(s, s);
+    (void)pt;
+    const bool want_pre = pre_q != nullptr && live;
+    const bool fast = (g.ys != 0.0f) & (ieee_only == 0) & (c0 + CW <= cend);
+    bool finite = true;   // every value quantized was finite
+    uint32_t cq[CW / PUB] = {};
+    // Column u of turn p; N live pairs. The update touches the pairs from the one that holds
+    // column u + 1 on (a value that is no longer read in a pair's lower half does no harm).
+    auto column = [&](auto exact_tag, auto live_tag, auto u_tag, int p, float& e, float& wpre, float& t, StepRange& sr) {
+        constexpr int N = decltype(live_tag)::value, u = decltype(u_tag)::value;
+        const int jj = PUB * p + u;
+        const float* rr = rt + jj * CW;
+        wpre = (u & 1) ? w[u / 2].y : w[u / 2].x;
+        column_step<decltype(exact_tag)::value>(wpre, g, rds[CW * s + jj], t, e, sr);
+        const float2 ne2 = make_float2(-e, -e), wp2 = make_float2(wpre, wpre);
+        (void)wp2;
+        constexpr int V0 = (u + 1) / 2;
+        constexpr int SH = u == PUB - 1 ? PUB / 2 : 0;
+#pragma unroll
+        for (int v = V0; v < N; ++v) {
+            float2 x = __ffma2_rn(ne2, *reinterpret_cast<const float2*>(rr + 2 * v), w[v]);
+            if constexpr (HASP) x = __ffma2_rn(wp2, *reinterpret_cast<const float2*>(pt + jj * CW + 2 * v), x);
+            w[v - SH] = x;
         }
-        if (!__all_sync(0xffffffffu, finite) && lane == 0) record_error(info, -KQ_ERR_NONFINITE);
+    };
+    auto columns = [&](auto exact_tag, auto live_tag, int p, float (&e)[PUB], float (&wpre)[PUB], float (&tq)[PUB], StepRange& sr) {
+        column(exact_tag, live_tag, std::integral_constant<int, 0>{}, p, e[0], wpre[0], tq[0], sr);
+        column(exact_tag, live_tag, std::integral_constant<int, 1>{}, p, e[1], wpre[1], tq[1], sr);
+        column(exact_tag, live_tag, std::integral_constant<int, 2>{}, p, e[2], wpre[2], tq[2], sr);
+        column(exact_tag, live_tag, std::integral_constant<int, 3>{}, p, e[3], wpre[3], tq[3], sr);
+    };
+    static_assert(PUB == 4, "columns() writes out the 4 columns of a turn");
+    const float czero = __fadd_rn(g.zero, 8388608.0f);   // t + czero = 2^23 + code
+#pragma unroll 1
+    for (int p = 0; p < CW / PUB; ++p) {
+        float e[PUB], wpre[PUB], tq[PUB];
+        StepRange sr;
+        // the columns left, in their own (not yet published) rows of the exchange tile
+#pragma unroll
+        for (int t = 0; t < CW / 2; ++t)
+            if (PUB * p + 2 * t < CW) {
+                xt[(PUB * p + 2 * t) * ELD + lane] = w[t].x;
+                xt[(PUB * p + 2 * t + 1) * ELD + lane] = w[t].y;
+            }
+        if (p < CW / PUB / 2)
+            columns(std::false_type{}, std::integral_constant<int, CW / 2>{}, p, e, wpre, tq, sr);
+        else
+            columns(std::false_type{}, std::integral_constant<int, CW / 4>{}, p, e, wpre, tq, sr);
+        uint32_t word = 0u;
+        if (__builtin_expect(sr.ok() & fast, 1)) {
+            uint32_t cb[PUB];
+#pragma unroll
+            for (int u = 0; u < PUB; ++u) {
+                xt[(PUB * p + u) * ELD + lane] = e[u];
+                if constexpr (HASP) Qs[s * XT + (PUB * p + u) * ELD + lane] = wpre[u];
+                cb[u] = __float_as_uint(__fadd_rn(tq[u], czero));
+            }
+            word = __byte_perm(__byte_perm(cb[0], cb[1], 0x0040), __byte_perm(cb[2], cb[3], 0x0040), 0x5410);
+            if (want_pre) {
+#pragma unroll
+                for (int u = 0; u < PUB; ++u)
+                    if (KQ_IN_RANGE(r * d_in + c0 + PUB * p + u, d_out * d_in)) pre_q[r * d_in + c0 + PUB * p + u] = wpre[u];
+            }
+        } else {   // an operand outside the fast division's range (or past the end): these columns again,
+                   // with IEEE divisions
+#pragma unroll
+            for (int t = 0; t < CW / 2; ++t)
+                if (PUB * p + 2 * t < CW)
+                    w[t] = make_float2(xt[(PUB * p + 2 * t) * ELD + lane], xt[(PUB * p + 2 * t + 1) * ELD + lane]);
+            columns(std::true_type{}, std::integral_constant<int, CW / 2>{}, p, e, wpre, tq, sr);
+#pragma unroll
+            for (int u = 0; u < PUB; ++u) {
+                const int jj = PUB * p + u;
+                xt[jj * ELD + lane] = e[u];
+                if constexpr (HASP) Qs[s * XT + jj * ELD + lane] = wpre[u];
+                word |= (__float_as_uint(__fadd_rn(tq[u], czero)) & 255u) << (8 * u);
+                finite = finite & ((fabsf(wpre[u]) <= 3.402823466e38f) | (CW * s + jj >= nb));
+                if (want_pre && c0 + jj < cend && KQ_IN_RANGE(r * d_in + c0 + jj, d_out * d_in)) pre_q[r * d_in + c0 + jj] = wpre[u];
+            }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&pub[s * (CW / PUB) + p]);
+#pragma unroll
+        for (int v = 0; v + 1 < CW / PUB; ++v) cq[v] = cq[v + 1];
+        cq[CW / PUB - 1] = word;
+    }
+    if (!__all_sync(0xffffffffu, finite) && lane == 0) record_error(info, -KQ_ERR_NONFINITE);
+    if (live && KQ_IN_RANGE(r * d_in + (c0 + CW <= cend ? c0 + CW : cend) - 1, d_out * d_in)) {
+        uint8_t* cp = codes + r * d_in + c0;
+        if (VEC && c0 + CW <= cend) {
+            *reinterpret_cast<uint4*>(cp) = make_uint4(cq[0], cq[1], cq[2], cq[3]);
+        } else {
+#pragma unroll
+            for (int t = 0; t < CW; ++t)
+                if (c0 + t < cend) cp[t] = static_cast<uint8_t>(cq[t >> 2] >> (8 * (t & 3)));
+        }
+    }
+    // E (and its tf32 split, and -Wpre) row by row from the exchange tile.
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+        const int64_t rr = row0 + 8 * it + qr;
+        float v[4], h[4], l[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = xt[(qc + u) * ELD + 8 * it + qr];
+        store_quad<VEC>(E, rr, d_out, d_in, c0 + qc, cend, v);
+        if (Eh) {   // tensor-core trailing update: E = E_hi + E_lo
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                h[u] = tf32_hi(v[u]);
+                l[u] = v[u] - h[u];
+            }
+            store_quad<VEC>(Eh, rr, d_out, d_in, c0 + qc, cend, h);
+            store_quad<VEC>(El, rr, d_out, d_in, c0 + qc, cend, l);
+        }
+        if constexpr (HASP) {   // -Wpre of the block, for the trailing update
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = -Qs[s * XT + (qc + u) * ELD + 8 * it + qr];
+            if (Qh) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    h[u] = tf32_hi(v[u]);
+                    l[u] = v[u] - h[u];
+                }
+                store_quad<VEC>(Qh, rr, d_out, d_in, c0 + qc, cend, h);
+                store_quad<VEC>(Ql, rr, d_out, d_in, c0 + qc, cend, l);
+            } else {
+                store_quad<VEC>(Q, rr, d_out, d_in, c0 + qc, cend, v);
+            }
+        }
     }
 }
 
@@ -737,17 +847,20 @@ extern "C" kq_status kq_obs_quantize(float* W, int64_t d_out, int64_t d_in, cons
     }
     static std::atomic<uint64_t> attr{0};
     KQ_TRY(once_per_device(attr, [&]() -> kq_status {
-        KQ_CUDA(cudaFuncSetAttribute(obs_block_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     OBS_SMEM_MMA));
-        KQ_CUDA(cudaFuncSetAttribute(obs_block_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     BLK * BLK * 4));
-        // Whole shared memory on the SM, so that a CTA fits beside a far-update CTA.
-        KQ_CUDA(cudaFuncSetAttribute(obs_block_kernel<true, false>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     cudaSharedmemCarveoutMaxShared));
-        KQ_CUDA(cudaFuncSetAttribute(obs_block_kernel<false, false>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     cudaSharedmemCarveoutMaxShared));
-        KQ_CUDA(cudaFuncSetAttribute(obs_block_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     2 * BLK * BLK * 4));
+        // The whole shared memory of the SM, so that a CTA fits beside a far-update CTA.
+        auto block_attr = [](auto* kern, bool with_p) -> kq_status {
+            KQ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, obs_smem(with_p)));
+            KQ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                         cudaSharedmemCarveoutMaxShared));
+            return KQ_OK;
+        };
+        KQ_TRY(block_attr(obs_block_kernel<true, false, FUSE_NONE>, false));
+        KQ_TRY(block_attr(obs_block_kernel<true, false, FUSE_NONE, 3>, false));
+        KQ_TRY(block_attr(obs_block_kernel<true, false, FUSE_FP32>, false));
+        KQ_TRY(block_attr(obs_block_kernel<true, false, FUSE_MMA>, false));
+        KQ_TRY(block_attr(obs_block_kernel<false, false, FUSE_NONE>, false));
+        KQ_TRY(block_attr(obs_block_kernel<false, false, FUSE_FP32>, false));
+        KQ_TRY(block_attr(obs_block_kernel<true, true, FUSE_NONE>, true));
         KQ_CUDA(cudaFuncSetAttribute(trailing_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      static_cast<int>(G_SMEM)));
         KQ_CUDA(cudaFuncSetAttribute(trailing_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -775,26 +888,24 @@ extern "C" kq_status kq_obs_quantize(float* W, int64_t d_out, int64_t d_in, cons
     const bool bvec = (d_in % 16 == 0) && (reinterpret_cast<uintptr_t>(W) % 16 == 0) &&
                       (reinterpret_cast<uintptr_t>(codes) % 16 == 0);
     const int64_t nblk = cdiv(d_in, BLK);
-    const int64_t row_ctas = hp ? std::min<int64_t>(cdiv(d_out, OBS_ROWS_P), static_cast<int64_t>(num_sms()))
-                                : std::min<int64_t>(cdiv(d_out, OBS_ROWS), 2 * static_cast<int64_t>(num_sms()));
-    pack_r_kernel<<<dim3(BLK / 32, BLK / 32, static_cast<unsigned>(nblk)), dim3(32, 8), 0, stream>>>(Lt, d_in, o.Rp, 0);
+    const int64_t row_ctas = cdiv(d_out, OBS_ROWS);
+    pack_r_kernel<<<dim3(RTILES, static_cast<unsigned>(nblk)), dim3(CW, CW), 0, stream>>>(Lt, d_in, o.Rp);
     KQ_LAUNCH_CHECK("pack_r_kernel");
-    // the blocks of R right of the diagonal ones, for the fused update: the tensor-core
-    // form's layout in the 3xTF32 mode, the block kernel's own otherwise
+    // the blocks of R right of the diagonal ones, for the fused update: as mma.sync fragments in
+    // the 3xTF32 mode, as rows otherwise
     const bool fuse_ok = !hp && nblk > 1 && row_ctas <= static_cast<int64_t>(num_sms()) &&
                          d_out * d_in <= (int64_t{24} << 20);
     const bool mma_fused = fuse_ok && tc && bvec;
-    if (fuse_ok && mma_fused) {
-        pack_rq_mma_kernel<<<dim3(BLK / 32, BLK / 32, static_cast<unsigned>(nblk - 1)), dim3(32, 8), 0, stream>>>(
-            Lt, d_in, o.Rq);
-        KQ_LAUNCH_CHECK("pack_rq_mma_kernel");
-    } else if (fuse_ok) {
-        pack_r_kernel<<<dim3(BLK / 32, BLK / 32, static_cast<unsigned>(nblk - 1)), dim3(32, 8), 0, stream>>>(Lt, d_in,
-                                                                                                          o.Rq, 1);
-        KQ_LAUNCH_CHECK("pack_r_kernel");
+    if (fuse_ok) {
+        const dim3 rqgrid(NWARP, static_cast<unsigned>(nblk - 1));
+        if (mma_fused)
+            pack_rq_kernel<true><<<rqgrid, 256, 0, stream>>>(Lt, d_in, o.Rq);
+        else
+            pack_rq_kernel<false><<<rqgrid, 256, 0, stream>>>(Lt, d_in, o.Rq);
+        KQ_LAUNCH_CHECK("pack_rq_kernel");
     }
     if (hp) {   // P[i0 + j][i0 + c] = Pt[i0 + c][i0 + j]: the same packing as R from Lt
-        pack_r_kernel<<<dim3(BLK / 32, BLK / 32, static_cast<unsigned>(nblk)), dim3(32, 8), 0, stream>>>(Pt, d_in, o.Pp, 0);
+        pack_r_kernel<<<dim3(RTILES, static_cast<unsigned>(nblk)), dim3(CW, CW), 0, stream>>>(Pt, d_in, o.Pp);
         KQ_LAUNCH_CHECK("pack_r_kernel");
     }
     // GPTQ mode: block b's kernel first applies the previous block's update of its own
@@ -829,22 +940,26 @@ extern "C" kq_status kq_obs_quantize(float* W, int64_t d_out, int64_t d_in, cons
         KQ_LAUNCH_CHECK("trailing_kernel");
         return KQ_OK;
     };
-    auto block_launch = [&](int64_t b, const float* rq) {
-        const int64_t i0 = b * BLK;
-        const float* rp = o.Rp + b * BLK * BLK;
-        if (hp)
-            obs_block_kernel<true, true><<<static_cast<unsigned>(row_ctas), OBS_THREADS_P, 2 * BLK * BLK * 4, stream>>>(
-                W, d_out, d_in, rp, i0, bits, group, o.gscale, o.gzero, codes, scale, zero, o.E, pre_q, o.Eh, o.El,
-                o.Pp + b * BLK * BLK, o.Q, o.Qh, o.Ql, nullptr, 0, info);
-        else if (bvec)
-            obs_block_kernel<true, false><<<static_cast<unsigned>(row_ctas), OBS_THREADS, mma_fused ? OBS_SMEM_MMA : BLK * BLK * 4,
-                                             stream>>>(
-                W, d_out, d_in, rp, i0, bits, group, o.gscale, o.gzero, codes, scale, zero, o.E, pre_q, o.Eh, o.El,
-                nullptr, nullptr, nullptr, nullptr, rq, mma_fused ? 1 : 0, info);
-        else
-            obs_block_kernel<false, false><<<static_cast<unsigned>(row_ctas), OBS_THREADS, BLK * BLK * 4, stream>>>(
-                W, d_out, d_in, rp, i0, bits, group, o.gscale, o.gzero, codes, scale, zero, o.E, pre_q, o.Eh, o.El,
-                nullptr, nullptr, nullptr, nullptr, rq, 0, info);
+    // `after_kernel`: the call before this one on the stream was a block kernel or a trailing
+    // update, and nothing was waited for in between. The kernel is then launched as its
+    // programmatic dependent: it stages R (packed before that kernel began) while the other
+    // drains. A block kernel lets its own dependent start only after its own wait, so
+    // everything before the kernel it depends on has finished.
+    auto block_launch = [&](int64_t b, const float* rq, bool after_kernel) -> kq_status {
+        auto go = [&](auto* kern) -> kq_status {
+            KQ_CUDA(launch_dependent(kern, dim3(static_cast<unsigned>(row_ctas)), dim3(OBS_THREADS), obs_smem(hp), stream, 1u,
+                                     after_kernel, W, d_out, d_in, o.Rp + b * RPACK, b * BLK, bits, group, o.gscale, o.gzero,
+                                     codes, scale, zero, o.E, pre_q, o.Eh, o.El, hp ? o.Pp + b * RPACK : nullptr, o.Q, o.Qh,
+                                     o.Ql, rq, info));
+            KQ_LAUNCH_CHECK("obs_block_kernel");
+            return KQ_OK;
+        };
+        if (hp) return go(obs_block_kernel<true, true, FUSE_NONE>);
+        // three CTAs per SM (80 registers, some 30 % more cycles a column) once two do not hold every row
+        if (!rq && bvec && row_ctas > 2 * static_cast<int64_t>(num_sms())) return go(obs_block_kernel<true, false, FUSE_NONE, 3>);
+        if (!rq) return bvec ? go(obs_block_kernel<true, false, FUSE_NONE>) : go(obs_block_kernel<false, false, FUSE_NONE>);
+        if (mma_fused) return go(obs_block_kernel<true, false, FUSE_MMA>);
+        return bvec ? go(obs_block_kernel<true, false, FUSE_FP32>) : go(obs_block_kernel<false, false, FUSE_FP32>);
     };
     // Two levels for the large layers on the tensor cores (super-panels of SPB blocks, the
     // GPTQ lazy update grouped once more): inside a super-panel each block updates the next
@@ -864,14 +979,13 @@ extern "C" kq_status kq_obs_quantize(float* W, int64_t d_out, int64_t d_in, cons
         cudaStream_t s_far = side ? side->s2 : stream;
         for (int64_t b = 0; b < nblk; ++b) {
             const int64_t i0 = b * BLK;
-            block_launch(b, nullptr);
-            KQ_LAUNCH_CHECK("obs_block_kernel");
+            kq_status st = block_launch(b, nullptr, b > 0);
+            if (st != KQ_OK) return st;
             const int64_t nb0 = i0 + BLK;                               // next block column
             if (nb0 >= d_in) break;
             const int64_t sp0 = (b / SPB) * SPW;                         // this super-panel
             const int64_t spe = std::min(d_in, sp0 + SPW);
             if (side) KQ_CUDA(cudaEventRecord(side->ev[0], stream));     // E of this block ready
-            kq_status st;
             if (nb0 < spe) {
                 if (in_pending) {   // it wrote the next block column too
                     KQ_CUDA(cudaStreamWaitEvent(stream, side->ev[1], 0));
@@ -930,8 +1044,8 @@ extern "C" kq_status kq_obs_quantize(float* W, int64_t d_out, int64_t d_in, cons
                 st = trailing(i0 - 2 * BLK, 2 * BLK, i0, std::min<int64_t>(d_in, i0 + 2 * BLK), stream);
                 if (st != KQ_OK) return st;
             }
-            block_launch(b, (b & 1) ? o.Rq + (b - 1) * BLK * BLK : nullptr);
-            KQ_LAUNCH_CHECK("obs_block_kernel");
+            st = block_launch(b, (b & 1) ? o.Rq + (b - 1) * BLK * BLK : nullptr, b > 0);
+            if (st != KQ_OK) return st;
             if ((b & 1) == 0) continue;
             const int64_t nb2 = std::min<int64_t>(d_in, i0 + 3 * BLK);   // beyond the next pair
             if (nb2 >= d_in) continue;
@@ -955,18 +1069,18 @@ extern "C" kq_status kq_obs_quantize(float* W, int64_t d_out, int64_t d_in, cons
             const int64_t b = i0 / BLK;
             const int kb = static_cast<int>(std::min<int64_t>(BLK, d_in - i0));
             const float* rq = fuse && b > 0 ? o.Rq + (b - 1) * BLK * BLK : nullptr;
-            if (fuse && far_pending[b & 1]) {   // the far update of block b - 2
+            const bool waits = fuse && far_pending[b & 1];
+            if (waits) {   // the far update of block b - 2
                 KQ_CUDA(cudaStreamWaitEvent(stream, side->ev2[b & 1], 0));
                 far_pending[b & 1] = false;
             }
-            block_launch(b, rq);
-            KQ_LAUNCH_CHECK("obs_block_kernel");
+            kq_status st = block_launch(b, rq, b > 0 && !waits);
+            if (st != KQ_OK) return st;
             const int64_t nb0 = i0 + kb;                                // next block column
             if (nb0 >= d_in) break;
             const int64_t nb1 = std::min<int64_t>(d_in, nb0 + BLK);    // columns beyond it: [nb1, d_in)
             const bool fork = side && nb1 < d_in;
             if (fork) KQ_CUDA(cudaEventRecord(side->ev[0], stream));           // E of this block ready
-            kq_status st;
             if (!fuse) {
                 if (forked) KQ_CUDA(cudaStreamWaitEvent(stream, side->ev[1], 0));  // previous far update done
                 st = trailing(i0, kb, nb0, nb1, stream);
