@@ -390,12 +390,12 @@ KQ_API kq_status kq_obs_quantize(float* W, int64_t d_out, int64_t d_in, const fl
  * kq_infer: y [B x d_out] fp32 = W^ x for B tokens x [B x d_in] fp32 (1 <= B <= 8), from
  *   the packed codes, scale fp32 and zero int32 ([d_out] for group 0, [d_out x d_in / 128]
  *   for group 128), s_x [d_in], s_g [d_out] and the RHT signs of the quantization.
- *   All arithmetic fp32 (codes are exact as floats; per group scale (sum q x' - zero sum x')).
+ *   fp32 throughout: the codes less the middle code are exact in bf16 and x' is the exact sum of
+ *   three bf16 terms, so the tensor cores' products are exact and summed in fp32 (per group
+ *   scale (sum (q - c) x' - (zero - c) sum x')).
  *   ws: kq_infer_workspace(B, d_in, d_out) bytes, 256-byte aligned. packed, x, y, s_x, s_g
  *   16-byte aligned, the signs 4-byte aligned, d_out % 4 == 0; s_x, s_g required (not NULL). d_in and d_out need Hadamard constructions (2^k or 28 * 2^k).
- *   info: optional device error word (see kq_check). The weight stream waits on its copies
- *   with a time limit; a wait that runs out records -KQ_ERR_TIMEOUT there and leaves that
- *   part of y as NaN.
+ *   info: optional device error word (see kq_check); no kernel of this call records in it.
  * ---------------------------------------------------------------------------------- */
 KQ_API size_t kq_packed_codes_bytes(int64_t d_out, int64_t d_in, int bits);
 KQ_API kq_status kq_pack_codes(const uint8_t* codes, int64_t d_out, int64_t d_in, int bits, uint32_t* packed,

@@ -939,11 +939,7 @@ extern "C" kq_status kq_rotate_out(float* W, int64_t d_out, int64_t d_in, float*
 
 // Used by the check-only revert (check.cu).
 namespace kq {
-// Used by the inference call (infer.cu): rows <- V S^-1 rows (pre-factor sigma / s).
-kq_status rotate_rows_pre_div(float* M, int64_t rows, int64_t n, const float* s, const int8_t* sign,
-                              cudaStream_t stream) {
-    return rows_transform(M, rows, n, s ? F_SDIV : F_SIGN, F_NONE, sign, s, stream);
-}
+// Used by the check-only revert (check.cu).
 kq_status rotate_rows_inv(float* M, int64_t rows, int64_t n, const float* s, const int8_t* sign,
                           cudaStream_t stream) {
     return rows_transform(M, rows, n, F_NONE, s ? F_SDIV : F_SIGN, sign, s, stream);
