@@ -16,6 +16,16 @@
 //     running sum held in registers (each thread owns 128 columns of one row), while the
 //     MMAs continue into the other accumulator. This bounds how many tensor-core
 //     additions any fp32 partial sum sees;
+//   * a factor with few tiles (a narrow d) leaves most SMs idle: a cluster of KS = 4 CTAs then
+//     shares each tile, CTA r taking the token chunks r, r + KS, ... and owning 128 / KS rows of
+//     the running sum. Each drained chunk goes to the owners' inboxes through distributed
+//     shared memory, and the owners add the chunks in token order, so H has the bits one CTA
+//     would give it. d = 1024, T = 262144 (20 tiles): 1384 -> 1047 us; d = 1400, T = 131072: 1134
+//     -> 620 us. What bounds it then is the exchange (~4 us a half tile: remote stores, their
+//     release, the owner's answer), so quarter tiles in two slots (1470 us) and clusters of two
+//     (d = 2048: 1597 against 1386 us) were slower. Splitting the columns instead (64 per CTA,
+//     the row panel multicast) took 1217 us at d = 1024: a CTA's time per 64 tokens is then bound
+//     by the bytes into its SM (50-70 per cycle) and the row operand, not by N;
 //   * every mbarrier wait is bounded (kq::mbar_wait); a timeout is reported as
 //     -KQ_ERR_TIMEOUT in *info and the CTA drains its own copies and MMAs before exit.
 #include <cstdio>
@@ -23,6 +33,7 @@
 #include <cstring>
 
 #include "kq_common.cuh"
+#include "trail_tc.cuh"
 
 namespace kq {
 namespace {
@@ -30,13 +41,16 @@ namespace {
 constexpr int BM = 128;   // output rows per tile (MMA M, TMEM lanes)
 constexpr int BN = 256;   // output columns per tile (MMA N)
 constexpr int BK = 64;    // tokens per pipeline stage
-constexpr int STAGES = 4;
 constexpr int BOX_BYTES = BK * 64 * 2;          // one 64-token x 64-feature bf16 box
 constexpr int A_BYTES = BK * BM * 2;            // 16 KB
 constexpr int B_BYTES = BK * BN * 2;            // 32 KB
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;  // 48 KB
 constexpr int NUM_THREADS = 320;                // 10 warps
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
+// Ring stages of a CTA, and its inbox when KS CTAs share a tile: per source CTA 128 / KS rows x 128
+// columns (half a tile at a time), 64 KB in all.
+__host__ __device__ constexpr int stages_of(int ks) { return ks == 1 ? 4 : 3; }
+constexpr int INBOX_BYTES = BM * 128 * 4;
+constexpr int smem_bytes(int ks) { return stages_of(ks) * STAGE_BYTES + (ks == 1 ? 0 : INBOX_BYTES) + 1024 + 256; }
 constexpr uint32_t TMEM_COLS = 512;
 // Canonical MN-major SW128 layout: atoms of 64 features x 8 tokens (1 KB). Along the MN
 // dimension atoms are one TMA box apart; along K they are 1 KB apart.
@@ -83,35 +97,46 @@ __device__ __forceinline__ bool wait_noabort(uint64_t* bar, uint32_t parity) {
     return mbar_wait(bar, parity, &dummy);
 }
 
+__device__ __forceinline__ void st_cluster_f4(uint32_t addr, float4 v) {
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+                 : "memory");
+}
+
 // The body shared by the two Gram products.
 //   CROSS = false (SYRK): H (+)= A^T A, lower 128 x 256 tiles mirrored on write-out; every
 //     operand box comes from map a0.
 //   CROSS = true: D (+)= (A_hi + A_lo)^T B over all tiles, no symmetry: the K loop runs over
 //     the T tokens of the pair (a0 = A_hi, b) and then over the pair (a1 = A_lo, b).
-template <bool CROSS>
+template <bool CROSS, int KS>
 __device__ __forceinline__ void gram_tc_body(const CUtensorMap* a0, const CUtensorMap* a1,
                                              const CUtensorMap* bmap, float* __restrict__ H, int d,
                                              int T, int n_row_tiles, int chunk_stages, int accumulate,
                                              int* info) {
+    constexpr int STAGES = stages_of(KS);
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
+    float* inbox = reinterpret_cast<float*>(smem + STAGES * STAGE_BYTES);   // KS > 1
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES + (KS > 1 ? INBOX_BYTES : 0));
     uint64_t* empty = full + STAGES;
     uint64_t* tfull = empty + STAGES;
     uint64_t* tempty = tfull + 2;
     uint64_t* mma_done = tempty + 2;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_done + 1);
+    uint64_t* in_full = mma_done + 1;     // [KS] a source's part of the inbox is there
+    uint64_t* in_free = in_full + KS;     // [KS] an owner has read this CTA's part of its inbox
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(in_free + KS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
+    const int tile = static_cast<int>(blockIdx.x) / KS;
+    const int rank = KS > 1 ? static_cast<int>(cluster_ctarank()) : 0;
     int ti, tj;
     if (CROSS) {
-        ti = static_cast<int>(blockIdx.x) % n_row_tiles;
-        tj = static_cast<int>(blockIdx.x) / n_row_tiles;
+        ti = tile % n_row_tiles;
+        tj = tile / n_row_tiles;
     } else {
-        tile_of(blockIdx.x, n_row_tiles, (d + BN - 1) / BN, &ti, &tj);
+        tile_of(tile, n_row_tiles, (d + BN - 1) / BN, &ti, &tj);
     }
     const int i0 = ti * BM;
     const int j0 = tj * BN;
@@ -129,6 +154,10 @@ __device__ __forceinline__ void gram_tc_body(const CUtensorMap* a0, const CUtens
             mbar_init(&tempty[b], 8);
         }
         mbar_init(mma_done, 1);
+        for (int r = 0; KS > 1 && r < KS; ++r) {
+            mbar_init(&in_full[r], 8 / KS);
+            mbar_init(&in_free[r], 8);
+        }
         *abort_flag = 0;
         fence_mbar_init();
     }
@@ -144,17 +173,21 @@ __device__ __forceinline__ void gram_tc_body(const CUtensorMap* a0, const CUtens
         }
     }
     tc_fence_before();
-    __syncthreads();
+    if constexpr (KS > 1)
+        cluster_barrier();   // every CTA's barriers are set up before another one signals them
+    else
+        __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    // This CTA's chunks c = rank, rank + KS, ..., its stages counted by ks (the ring position).
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
         if (lane == 0) {
             int issued = 0;
-            for (int k = 0; k < nk; ++k) {
-                const int s = k % STAGES;
-                const uint32_t u = static_cast<uint32_t>(k / STAGES);
+            for (int k = rank * chunk_stages; k < nk; k += (KS > 1 && (k + 1) % chunk_stages == 0) ? (KS - 1) * chunk_stages + 1 : 1) {
+                const int s = issued % STAGES;
+                const uint32_t u = static_cast<uint32_t>(issued / STAGES);
                 if (!mbar_wait(&empty[s], (u & 1u) ^ 1u, abort_flag)) break;
                 mbar_arrive_expect_tx(&full[s], STAGE_BYTES);
                 uint8_t* a = smem + s * STAGE_BYTES;
@@ -168,7 +201,7 @@ __device__ __forceinline__ void gram_tc_body(const CUtensorMap* a0, const CUtens
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
                     tma_load_2d(b + q * BOX_BYTES, bm, &full[s], j0 + 64 * q, y);
-                issued = k + 1;
+                ++issued;
             }
             // Drain: every issued load must have landed before the CTA may exit.
             for (int k = (issued > STAGES ? issued - STAGES : 0); k < issued; ++k)
@@ -178,16 +211,16 @@ __device__ __forceinline__ void gram_tc_body(const CUtensorMap* a0, const CUtens
         // ------------------------------------------------------------ MMA issuer
         if (lane == 0) {
             constexpr uint32_t idesc = idesc_bf16_mn_major(BM, BN);
-            int k = 0;
+            int k = 0;   // stages of this CTA so far
             bool ok = true;
-            for (int c = 0; c < nchunks && ok; ++c) {
-                const int buf = c & 1;
-                const uint32_t u = static_cast<uint32_t>(c >> 1);
+            for (int c = rank, m = 0; c < nchunks && ok; c += KS, ++m) {
+                const int buf = m & 1;
+                const uint32_t u = static_cast<uint32_t>(m >> 1);
                 if (!mbar_wait(&tempty[buf], (u & 1u) ^ 1u, abort_flag)) break;
                 tc_fence_after();
                 const uint32_t dt = tmem + static_cast<uint32_t>(buf * BN);
-                const int kend = min(nk, (c + 1) * chunk_stages);
-                for (int kk = 0; k < kend; ++k, ++kk) {
+                const int kn = min(nk - c * chunk_stages, chunk_stages);
+                for (int kk = 0; kk < kn; ++k, ++kk) {
                     const int s = k % STAGES;
                     if (!mbar_wait(&full[s], static_cast<uint32_t>(k / STAGES) & 1u, abort_flag)) {
                         ok = false;
@@ -210,7 +243,7 @@ __device__ __forceinline__ void gram_tc_body(const CUtensorMap* a0, const CUtens
             tc_commit(mma_done);
             wait_noabort(mma_done, 0);
         }
-    } else {
+    } else if constexpr (KS == 1) {
         // ------------------------------------------------------------ epilogue (8 warps)
         const int q = warp & 3;                 // TMEM lane quadrant this warp may access
         const int half = (warp - 2) >> 2;       // which 128 of the 256 columns
@@ -292,9 +325,145 @@ __device__ __forceinline__ void gram_tc_body(const CUtensorMap* a0, const CUtens
                 }
             }
         }
+    } else {
+        // --------------------------------------------- epilogue of a shared tile (8 warps)
+        // Round m: this CTA's chunk (c = KS m + rank) goes to the owners' inboxes, 128 columns at a
+        // time, the warp's 32 TMEM lanes to the owner of those rows; then the owners' warps add the
+        // round's chunks in order, each thread 16 / KS float4 of its CTA's rows. Inbox of a source:
+        // [column quad 32][row 128 / KS] float4.
+        constexpr int RO = BM / KS;             // rows owned
+        constexpr int QN = RO / 32;             // quadrants (32-row groups) owned
+        const int w = warp - 2;
+        const int q = warp & 3;                 // TMEM lane quadrant this warp may access
+        const int half = w >> 2;                // which 64 of a phase's 128 columns
+        const int owner = q / QN;
+        float4 acc[2][4 * QN];                  // [phase][quad of columns 4 w + .., row group]
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int i = 0; i < 4 * QN; ++i) acc[h][i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        const uint32_t box = smem_u32(inbox) + static_cast<uint32_t>(rank * RO * 128 * 4);   // my part of any owner's inbox
+        const uint32_t box_at = mapa_shared(box, static_cast<uint32_t>(owner)) +
+                                static_cast<uint32_t>(((half * 16) * RO + (q % QN) * 32 + lane) * 16);
+        const uint32_t full_at = mapa_shared(smem_u32(&in_full[rank]), static_cast<uint32_t>(owner));
+        bool ok = true;
+        const int rounds = (nchunks + KS - 1) / KS;
+        for (int m = 0; m < rounds && ok; ++m) {
+            const bool mine = m * KS + rank < nchunks;
+            const int buf = m & 1;
+            if (mine) {
+                ok = mbar_wait(&tfull[buf], static_cast<uint32_t>(m >> 1) & 1u, abort_flag);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tc_fence_after();
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t ph = static_cast<uint32_t>(2 * m + h);
+                if (mine) {
+                    // the owner has added this CTA's previous part (the first wait passes at once)
+                    ok = mbar_wait_cl(&in_free[owner], (ph & 1u) ^ 1u, abort_flag);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    const uint32_t base = tmem + (static_cast<uint32_t>(q * 32) << 16) +
+                                          static_cast<uint32_t>(buf * BN + h * 128 + half * 64);
+#pragma unroll
+                    for (int p = 0; p < 2; ++p) {
+                        float v[32];
+                        tmem_ld32(base + p * 32, v);
+                        tc_wait_ld();
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            st_cluster_f4(box_at + static_cast<uint32_t>((p * 8 + i) * RO * 16),
+                                          make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
+                    }
+                    if (h == 1) tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) {
+                        mbar_arrive_remote(full_at);
+                        if (h == 1) mbar_arrive(&tempty[buf]);
+                    }
+                }
+                for (int src = 0; src < KS && ok; ++src) {
+                    if (m * KS + src >= nchunks) break;
+                    ok = mbar_wait_cl(&in_full[src], ph & 1u, abort_flag);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    const float4* in = reinterpret_cast<const float4*>(inbox) + src * RO * 32 + 4 * w * RO + lane;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int g = 0; g < QN; ++g) {
+                            const float4 v = in[i * RO + 32 * g];
+                            float4& a = acc[h][i * QN + g];
+                            a.x += v.x;
+                            a.y += v.y;
+                            a.z += v.z;
+                            a.w += v.w;
+                        }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_remote(mapa_shared(smem_u32(&in_free[rank]), static_cast<uint32_t>(src)));
+                }
+            }
+        }
+        // Write-out of the owned rows through shared memory (ring and inbox are idle: every chunk
+        // sent here has been added), coalesced in both triangles as above.
+        ok = named_bar_all(1, 256, ok && !*abort_flag);
+        if (ok) {
+            constexpr int SLD = BN + 1;
+            float* st = reinterpret_cast<float*>(smem);
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int g = 0; g < QN; ++g) {
+                        float* x = st + (32 * g + lane) * SLD + 128 * h + 16 * w + 4 * i;
+                        const float4 v = acc[h][i * QN + g];
+                        x[0] = v.x;
+                        x[1] = v.y;
+                        x[2] = v.z;
+                        x[3] = v.w;
+                    }
+            named_bar_all(1, 256, true);
+            const int rbase = i0 + rank * RO;
+#pragma unroll 2
+            for (int r = w; r < RO; r += 8) {
+                const int rr = rbase + r;
+                float old[8];
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    const int col = j0 + lane + 32 * t;
+                    old[t] = (accumulate && rr < d && col < d && (CROSS || col <= rr)) ? H[static_cast<int64_t>(rr) * d + col] : 0.0f;
+                }
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    const int col = j0 + lane + 32 * t;
+                    if (rr < d && col < d && (CROSS || col <= rr) &&
+                        KQ_IN_RANGE(static_cast<int64_t>(rr) * d + col, static_cast<int64_t>(d) * d)) {
+                        const float v = st[r * SLD + lane + 32 * t] + old[t];
+                        H[static_cast<int64_t>(rr) * d + col] = v;
+                        st[r * SLD + lane + 32 * t] = v;
+                    }
+                }
+            }
+            named_bar_all(1, 256, true);
+            if (!CROSS) {
+#pragma unroll 4
+                for (int e = w; e < BN * QN; e += 8) {
+                    const int col = j0 + e / QN, r = 32 * (e % QN) + lane, rr = rbase + r;
+                    if (rr < d && col < d && col < rr && KQ_IN_RANGE(static_cast<int64_t>(col) * d + rr, static_cast<int64_t>(d) * d))
+                        H[static_cast<int64_t>(col) * d + rr] = st[r * SLD + e / QN];
+                }
+            }
+        }
     }
 
-    __syncthreads();
+    // (of a cluster: no CTA leaves while another one may still write to it or signal it)
+    if constexpr (KS > 1)
+        cluster_barrier();
+    else
+        __syncthreads();
     if (*abort_flag && threadIdx.x == 0) record_error(info, -KQ_ERR_TIMEOUT);
     if (warp == 1) {
         tc_fence_after();
@@ -302,18 +471,23 @@ __device__ __forceinline__ void gram_tc_body(const CUtensorMap* a0, const CUtens
     }
 }
 
+template <int KS>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 syrk_tc_kernel(const __grid_constant__ CUtensorMap tmap, float* __restrict__ H, int d, int T,
                int n_row_tiles, int chunk_stages, int accumulate, int* info) {
-    gram_tc_body<false>(&tmap, &tmap, &tmap, H, d, T, n_row_tiles, chunk_stages, accumulate, info);
+    gram_tc_body<false, KS>(&tmap, &tmap, &tmap, H, d, T, n_row_tiles, chunk_stages, accumulate, info);
 }
 
+template <int KS>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 drift_tc_kernel(const __grid_constant__ CUtensorMap a_hi, const __grid_constant__ CUtensorMap a_lo,
                 const __grid_constant__ CUtensorMap b, float* __restrict__ D, int d, int T,
                 int n_row_tiles, int chunk_stages, int accumulate, int* info) {
-    gram_tc_body<true>(&a_hi, &a_lo, &b, D, d, T, n_row_tiles, chunk_stages, accumulate, info);
+    gram_tc_body<true, KS>(&a_hi, &a_lo, &b, D, d, T, n_row_tiles, chunk_stages, accumulate, info);
 }
+
+// CTAs that share a tile: four while all of them still run at once (one per SM) and each has a chunk.
+int ks_of(int64_t tiles, int64_t chunks) { return 4 * tiles <= num_sms() && chunks >= 4 ? 4 : 1; }
 
 // Round a finite fp32 value to the nearest bf16, ties to even; returns the 16 bf16 bits.
 __device__ __forceinline__ uint32_t bf16_rn_bits(float f) {
@@ -455,18 +629,23 @@ extern "C" kq_status kq_accum_factor(const uint16_t* A, int64_t T, int64_t d, in
         if (st != KQ_OK) return st;
         static std::atomic<uint64_t> attr_set{0};
         KQ_TRY(once_per_device(attr_set, [&]() -> kq_status {
-            KQ_CUDA(cudaFuncSetAttribute(syrk_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         SMEM_BYTES));
+            KQ_CUDA(cudaFuncSetAttribute(syrk_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(1)));
+            KQ_CUDA(cudaFuncSetAttribute(syrk_tc_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(4)));
             return KQ_OK;
         }));
         const int n_row = static_cast<int>(cdiv(d, BM));
         const int n_col = static_cast<int>(cdiv(d, BN));
         int64_t tiles = 0;
         for (int j = 0; j < n_col; ++j) tiles += (n_row - 2 * j > 0) ? n_row - 2 * j : 0;
-        const int chunk_stages = syrk_chunk_stages();
-        syrk_tc_kernel<<<static_cast<unsigned>(tiles), NUM_THREADS, SMEM_BYTES, stream>>>(
-            tmap, H, static_cast<int>(d), static_cast<int>(T), n_row, chunk_stages, accumulate, info);
-        KQ_LAUNCH_CHECK("syrk_tc_kernel");
+        const int ks = ks_of(tiles, cdiv(T, KQ_SYRK_CHUNK_TOKENS));
+        auto go = [&](auto* kern) -> kq_status {
+            KQ_CUDA(launch_dependent(kern, dim3(static_cast<unsigned>(tiles * ks)), dim3(NUM_THREADS), smem_bytes(ks), stream,
+                                     static_cast<unsigned>(ks), false, tmap, H, static_cast<int>(d), static_cast<int>(T),
+                                     n_row, syrk_chunk_stages(), accumulate, info));
+            KQ_LAUNCH_CHECK("syrk_tc_kernel");
+            return KQ_OK;
+        };
+        KQ_TRY(ks == 4 ? go(syrk_tc_kernel<4>) : go(syrk_tc_kernel<1>));
     }
     if (trace) return launch_trace(H, d, trace, stream);
     return KQ_OK;
@@ -512,12 +691,12 @@ extern "C" kq_status kq_accum_drift(const uint16_t* Xt, const uint16_t* X, int64
     uint16_t* lo = hi + Tc * d;
     static std::atomic<uint64_t> attr_set{0};
     KQ_TRY(once_per_device(attr_set, [&]() -> kq_status {
-        KQ_CUDA(cudaFuncSetAttribute(drift_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+        KQ_CUDA(cudaFuncSetAttribute(drift_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(1)));
+        KQ_CUDA(cudaFuncSetAttribute(drift_tc_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(4)));
         return KQ_OK;
     }));
     const int n_row = static_cast<int>(cdiv(d, BM));
     const int n_col = static_cast<int>(cdiv(d, BN));
-    const int chunk_stages = syrk_chunk_stages();
     for (int64_t t0 = 0; t0 < T; t0 += Tc) {
         const int64_t tn = std::min<int64_t>(Tc, T - t0);
         const int64_t vecs = tn * (d / 8);
@@ -530,10 +709,15 @@ extern "C" kq_status kq_accum_drift(const uint16_t* Xt, const uint16_t* X, int64
         if (st == KQ_OK) st = make_bf16_map(&ml, lo, d, tn, d, "kq_accum_drift");
         if (st == KQ_OK) st = make_bf16_map(&mb, X + t0 * ld, d, tn, ld, "kq_accum_drift");
         if (st != KQ_OK) return st;
-        drift_tc_kernel<<<static_cast<unsigned>(n_row * n_col), NUM_THREADS, SMEM_BYTES, stream>>>(
-            mh, ml, mb, D, static_cast<int>(d), static_cast<int>(tn), n_row, chunk_stages,
-            (accumulate || t0 > 0) ? 1 : 0, info);
-        KQ_LAUNCH_CHECK("drift_tc_kernel");
+        const int ks = ks_of(static_cast<int64_t>(n_row) * n_col, cdiv(2 * cdiv(tn, BK), syrk_chunk_stages()));
+        auto go = [&](auto* kern) -> kq_status {
+            KQ_CUDA(launch_dependent(kern, dim3(static_cast<unsigned>(n_row * n_col * ks)), dim3(NUM_THREADS), smem_bytes(ks),
+                                     stream, static_cast<unsigned>(ks), false, mh, ml, mb, D, static_cast<int>(d),
+                                     static_cast<int>(tn), n_row, syrk_chunk_stages(), (accumulate || t0 > 0) ? 1 : 0, info));
+            KQ_LAUNCH_CHECK("drift_tc_kernel");
+            return KQ_OK;
+        };
+        KQ_TRY(ks == 4 ? go(drift_tc_kernel<4>) : go(drift_tc_kernel<1>));
     }
     return KQ_OK;
 }
