@@ -154,21 +154,26 @@ __global__ void prep4_kernel(const float* __restrict__ H, int64_t n, int64_t npa
 // u = w / d; a block-row column x (left of the block) gives h = L_b^-1 x; the four scalar
 // updates of a below-block entry sum to M_ik -= sum_t u_i^t h_k^t with h = w for columns
 // right of the block. Panel entries end as w_s - sum_{t>s} u^t b_ts, block-row entries as
-// h, and the pivot block as b. The pivot block's owner factors it once and publishes the
-// record; panel rows and block-row rows are published raw by their owners. One barrier
-// per block column; the staging is double-buffered.
+// h, and the pivot block as b.
 //
-// Thread t < 528 owns one 4 x 4 block of the lower triangle (row-major block order) in
-// registers. Pivots are checked by thread 0 (first non-positive one reported).
-constexpr int DIAG_THREADS = 544;                            // 528 owners + 16 idle lanes
-constexpr int DG_OWNERS = (NB / 4) * (NB / 4 + 1) / 2;       // 528
-constexpr int DG_PIV = 32;                                   // floats per pivot record
-constexpr size_t DIAG_SMEM =
-    (2 * NB * 4 + 2 * 4 * NB + 2 * DG_PIV + NB) * sizeof(float);
-
-struct Piv4 {   // factored 4 x 4 pivot block: 1 / d, unit-lower L_b, raw inverse rows b
-    float rd[4], l10, l20, l30, l21, l31, l32, b10, b20, b30, b21, b31, b32;
-};
+// Per block column two barriers: 128 threads solve one vector each (a panel row: w and u; a
+// block-row column: h), then every owner below the pivot row updates its block from four rows
+// of u and of h, in packed pairs (f32x2 fma: the same roundings), and the next pivot's raw row and
+// column and its factored record are published. A panel block takes the same update with m = w
+// and h = b (the strictly lower inverse block of the pivot; its zeros change nothing). The
+// solved rows stay in shared memory (64 KB) and are scaled and written at the end.
+// Bound: the chain barrier - solve - barrier - update - factor of the next pivot (four dependent
+// reciprocals), so warp 0 holds the 32 diagonal blocks, one per lane, and nothing else; threads
+// 32 .. 527 own the 4 x 4 blocks below the diagonal in registers, row by row (finished rows leave
+// whole warps idle), threads 32 .. 159 solve.
+// 128 x 128 block, one CTA: 24.7 us; 32 us with every block solving its own row and column
+// vectors and panel, row and pivot owners spread over all warps.
+constexpr int DIAG_THREADS = 544;                            // 32 diagonal + 496 other owners + 16 idle lanes
+constexpr int DG_BELOW = (NB / 4) * (NB / 4 - 1) / 2;        // 496
+constexpr int DG_PIV = 12;                                   // floats of the pivot record: 1 / d, l, pad
+constexpr int DG_HIST = (NB / 4) * 4 * NB;                   // solved rows of every block step
+constexpr int DG_BM = (NB / 4) * 16;                         // strictly lower b of every pivot block
+constexpr size_t DIAG_SMEM = (DG_HIST + DG_BM + 3 * 4 * NB + DG_PIV + 3 * NB) * sizeof(float);
 
 __device__ __forceinline__ float rcp_approx(float x) {
     float r;
@@ -176,239 +181,189 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return r;
 }
 
-// x <- L_b^-1 x
-__device__ __forceinline__ void unit_lower_solve(float& x0, float& x1, float& x2, float& x3, const Piv4& p) {
-    x1 = fmaf(-p.l10, x0, x1);
-    x2 = fmaf(-p.l20, x0, x2);
-    x3 = fmaf(-p.l30, x0, x3);
-    x2 = fmaf(-p.l21, x1, x2);
-    x3 = fmaf(-p.l31, x1, x3);
-    x3 = fmaf(-p.l32, x2, x3);
+// The pivot block of a step, raw in m: its factored record to Pv (1 / d, l) and dv (d); m becomes
+// the strictly lower inverse rows b, which diag_store_b writes beside the next solve.
+__device__ __forceinline__ void diag_factor(float2 (&m)[4][2], float* Pv, float* dv) {
+    float a11 = m[1][0].y, a21 = m[2][0].y, a31 = m[3][0].y, a22 = m[2][1].x, a32 = m[3][1].x, a33 = m[3][1].y;
+    const float d0 = m[0][0].x, g10 = m[1][0].x, g20 = m[2][0].x, g30 = m[3][0].x;
+    const float r0 = rcp_approx(d0);
+    const float l10 = g10 * r0, l20 = g20 * r0, l30 = g30 * r0;
+    a11 = fmaf(-l10, g10, a11);
+    a21 = fmaf(-l20, g10, a21);
+    a31 = fmaf(-l30, g10, a31);
+    a22 = fmaf(-l20, g20, a22);
+    a32 = fmaf(-l30, g20, a32);
+    a33 = fmaf(-l30, g30, a33);
+    const float d1 = a11, g21 = a21, g31 = a31;
+    const float r1 = rcp_approx(d1);
+    const float l21 = g21 * r1, l31 = g31 * r1;
+    a22 = fmaf(-l21, g21, a22);
+    a32 = fmaf(-l31, g21, a32);
+    a33 = fmaf(-l31, g31, a33);
+    const float d2 = a22, g32 = a32;
+    const float r2 = rcp_approx(d2);
+    const float l32 = g32 * r2;
+    a33 = fmaf(-l32, g32, a33);
+    const float d3 = a33;
+    const float r3 = rcp_approx(d3);
+    *reinterpret_cast<float4*>(Pv) = make_float4(r0, r1, r2, r3);
+    *reinterpret_cast<float4*>(Pv + 4) = make_float4(l10, l20, l30, l21);
+    *reinterpret_cast<float2*>(Pv + 8) = make_float2(l31, l32);
+    *reinterpret_cast<float4*>(dv) = make_float4(d0, d1, d2, d3);
+    const float b20 = fmaf(-l21, g10, g20);
+    const float b31 = fmaf(-l32, g21, g31);
+    const float b30 = fmaf(-l32, b20, fmaf(-l31, g10, g30));
+    m[1][0].x = g10;
+    m[2][0] = make_float2(b20, g21);
+    m[3][0] = make_float2(b30, b31);
+    m[3][1].x = g32;
+}
+__device__ __forceinline__ void diag_store_b(const float2 (&m)[4][2], float* Bm) {
+    *reinterpret_cast<float4*>(Bm) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    *reinterpret_cast<float4*>(Bm + 4) = make_float4(m[1][0].x, 0.0f, 0.0f, 0.0f);
+    *reinterpret_cast<float4*>(Bm + 8) = make_float4(m[2][0].x, m[2][0].y, 0.0f, 0.0f);
+    *reinterpret_cast<float4*>(Bm + 12) = make_float4(m[3][0].x, m[3][0].y, m[3][1].x, 0.0f);
 }
 
-// Publish the inputs of block step q (buffer q & 1): block-row rows (left of the pivot),
-// panel rows (below it), and the factored pivot, whose owner also sets its block final.
-__device__ __forceinline__ void diag_publish(int q, float (&m)[4][4], int bi, int bk, float* Pst, float* Qst,
-                                             float* Pv) {
-    const int buf = q & 1;
-    const int i0 = 4 * bi, k0 = 4 * bk;
-    if (bi == q && bk < q) {
+// The raw inputs of block step q from a block below the diagonal: block-row columns (left of the
+// pivot) and panel rows (below it), one 4-vector per index.
+__device__ __forceinline__ void diag_publish(int q, const float2 (&m)[4][2], int bi, int bk, float* Raw) {
+    if (bi == q) {
+        float* x = Raw + 16 * bk;   // columns 4 bk .. + 3: rows t of the block
+        *reinterpret_cast<float4*>(x) = make_float4(m[0][0].x, m[1][0].x, m[2][0].x, m[3][0].x);
+        *reinterpret_cast<float4*>(x + 4) = make_float4(m[0][0].y, m[1][0].y, m[2][0].y, m[3][0].y);
+        *reinterpret_cast<float4*>(x + 8) = make_float4(m[0][1].x, m[1][1].x, m[2][1].x, m[3][1].x);
+        *reinterpret_cast<float4*>(x + 12) = make_float4(m[0][1].y, m[1][1].y, m[2][1].y, m[3][1].y);
+    }
+    if (bk == q) {
 #pragma unroll
         for (int r = 0; r < 4; ++r)
-            *reinterpret_cast<float4*>(Qst + buf * 4 * NB + r * NB + k0) = make_float4(m[r][0], m[r][1], m[r][2], m[r][3]);
-    }
-    if (bk == q && bi > q) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-            *reinterpret_cast<float4*>(Pst + buf * NB * 4 + (i0 + r) * 4) = make_float4(m[r][0], m[r][1], m[r][2], m[r][3]);
-    }
-    if (bi == q && bk == q) {
-        float a11 = m[1][1], a21 = m[2][1], a31 = m[3][1], a22 = m[2][2], a32 = m[3][2], a33 = m[3][3];
-        const float d0 = m[0][0], g10 = m[1][0], g20 = m[2][0], g30 = m[3][0];
-        const float r0 = rcp_approx(d0);
-        const float l10 = g10 * r0, l20 = g20 * r0, l30 = g30 * r0;
-        a11 = fmaf(-l10, g10, a11);
-        a21 = fmaf(-l20, g10, a21);
-        a31 = fmaf(-l30, g10, a31);
-        a22 = fmaf(-l20, g20, a22);
-        a32 = fmaf(-l30, g20, a32);
-        a33 = fmaf(-l30, g30, a33);
-        const float d1 = a11, g21 = a21, g31 = a31;
-        const float r1 = rcp_approx(d1);
-        const float l21 = g21 * r1, l31 = g31 * r1;
-        a22 = fmaf(-l21, g21, a22);
-        a32 = fmaf(-l31, g21, a32);
-        a33 = fmaf(-l31, g31, a33);
-        const float d2 = a22, g32 = a32;
-        const float r2 = rcp_approx(d2);
-        const float l32 = g32 * r2;
-        a33 = fmaf(-l32, g32, a33);
-        const float d3 = a33;
-        const float r3 = rcp_approx(d3);
-        const float b10 = g10, b21 = g21, b32 = g32;
-        const float b20 = fmaf(-l21, b10, g20);
-        const float b31 = fmaf(-l32, b21, g31);
-        const float b30 = fmaf(-l32, b20, fmaf(-l31, b10, g30));
-        float* pv = Pv + buf * DG_PIV;
-        *reinterpret_cast<float4*>(pv) = make_float4(r0, r1, r2, r3);
-        *reinterpret_cast<float4*>(pv + 4) = make_float4(l10, l20, l30, l21);
-        *reinterpret_cast<float4*>(pv + 8) = make_float4(l31, l32, b10, b20);
-        *reinterpret_cast<float4*>(pv + 12) = make_float4(b30, b21, b31, b32);
-        *reinterpret_cast<float4*>(pv + 16) = make_float4(d0, d1, d2, d3);
-        m[1][0] = b10;
-        m[2][0] = b20;
-        m[3][0] = b30;
-        m[2][1] = b21;
-        m[3][1] = b31;
-        m[3][2] = b32;
+            *reinterpret_cast<float4*>(Raw + 16 * bi + 4 * r) = make_float4(m[r][0].x, m[r][0].y, m[r][1].x, m[r][1].y);
     }
 }
 
 __global__ void __launch_bounds__(DIAG_THREADS) chol_diag_kernel(Work w, int64_t n, int64_t npad, int k, int* info) {
     extern __shared__ __align__(16) float sm[];
-    float* Pst = sm;                      // [2][NB][4]   panel rows
-    float* Qst = Pst + 2 * NB * 4;        // [2][4][NB]   block-row rows
-    float* Pv = Qst + 2 * 4 * NB;         // [2][DG_PIV]  pivot records
-    float* dv = Pv + 2 * DG_PIV;          // [NB]         pivots d
+    float* Hist = sm;                     // [NB / 4][4][NB]  per step: h of the columns, w of the panel rows
+    float* Bm = Hist + DG_HIST;           // [NB / 4][4][4]   b of every pivot block
+    float* Raw = Bm + DG_BM;              // [NB][4]  raw vectors of the step
+    float* U = Raw + 4 * NB;              // [NB][4]  -u of the panel rows
+    float* Wr = U + 4 * NB;               // [NB][4]  w of the panel rows
+    float* Pv = Wr + 4 * NB;              // pivot record
+    float* dv = Pv + DG_PIV;              // [NB]     pivots d
+    float* isq = dv + NB;
+    float* idv = isq + NB;
+    __shared__ int first_bad;             // first non-positive pivot
     const int tid = threadIdx.x;
+    if (tid == 0) first_bad = NB;
     const int64_t off = static_cast<int64_t>(k) * NB;
-    const bool owner = tid < DG_OWNERS;
-    int bi = 0, bk = 0;
-    if (owner) {
-        int rem = tid;
-        while (rem > bi) {
-            rem -= bi + 1;
+    const bool diag = tid < 32;
+    int bi = tid, bk = tid;
+    if (!diag) {
+        int rem = tid - 32;
+        bi = 1;
+        while (rem >= bi && bi < NB / 4) {
+            rem -= bi;
             ++bi;
         }
         bk = rem;
     }
+    const bool owner = bi < NB / 4;   // the last 16 threads own nothing
     const int i0 = 4 * bi, k0 = 4 * bk;
-    float m[4][4];
+    float2 m[4][2] = {};
     if (owner) {
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             const float4 v = *reinterpret_cast<const float4*>(w.A + (off + i0 + r) * npad + off + k0);
-            m[r][0] = v.x;
-            m[r][1] = v.y;
-            m[r][2] = v.z;
-            m[r][3] = v.w;
+            m[r][0] = make_float2(v.x, v.y);
+            m[r][1] = make_float2(v.z, v.w);
         }
-        diag_publish(0, m, bi, bk, Pst, Qst, Pv);
+        if (tid == 0) diag_factor(m, Pv, dv);
+        if (!diag) diag_publish(0, m, bi, bk, Raw);
     }
     __syncthreads();
 #pragma unroll 1
     for (int q = 0; q < NB / 4; ++q) {
-        const int buf = q & 1;
-        const float* pv = Pv + buf * DG_PIV;
-        if (tid == 0) {
+        float* Hq = Hist + q * 4 * NB;
+        const int x = tid - 32;
+        if (x >= 0 && x < NB && (x >> 2) != q) {   // x <- L_b^-1 x, and u = x / d for a panel row
+            const float4 rd = *reinterpret_cast<const float4*>(Pv);
+            const float4 l = *reinterpret_cast<const float4*>(Pv + 4);    // l10 l20 l30 l21
+            const float2 l2 = *reinterpret_cast<const float2*>(Pv + 8);   // l31 l32
+            float4 v = *reinterpret_cast<const float4*>(Raw + 4 * x);
+            v.y = fmaf(-l.x, v.x, v.y);
+            v.z = fmaf(-l.y, v.x, v.z);
+            v.w = fmaf(-l.z, v.x, v.w);
+            v.z = fmaf(-l.w, v.y, v.z);
+            v.w = fmaf(-l2.x, v.y, v.w);
+            v.w = fmaf(-l2.y, v.z, v.w);
+            Hq[x] = v.x;
+            Hq[NB + x] = v.y;
+            Hq[2 * NB + x] = v.z;
+            Hq[3 * NB + x] = v.w;
+            *reinterpret_cast<float4*>(U + 4 * x) = make_float4(-(v.x * rd.x), -(v.y * rd.y), -(v.z * rd.z), -(v.w * rd.w));
+            *reinterpret_cast<float4*>(Wr + 4 * x) = v;
+        }
+        if (tid == q) diag_store_b(m, Bm + 16 * q);
+        __syncthreads();
+        if (bi > q && owner) {
+            float2 h[4][2];
+            float4 u[4];
+            const float* hp = bk == q ? Bm + 16 * q : Hq + k0;
+            const int hs = bk == q ? 4 : NB;
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
-                const float d = pv[16 + t];
-                dv[4 * q + t] = d;
-                if (!(d > 0.0f)) {
-                    const int64_t rev = off + 4 * q + t;
-                    if (rev < n) record_error(info, static_cast<int>(n - rev));
-                }
+                const float4 v = *reinterpret_cast<const float4*>(hp + t * hs);
+                h[t][0] = make_float2(v.x, v.y);
+                h[t][1] = make_float2(v.z, v.w);
             }
-        }
-        if (owner && bi >= q && !(bi == q && bk >= q)) {
-            Piv4 p;
-            {
-                const float4 v0 = *reinterpret_cast<const float4*>(pv);
-                const float4 v1 = *reinterpret_cast<const float4*>(pv + 4);
-                const float4 v2 = *reinterpret_cast<const float4*>(pv + 8);
-                const float4 v3 = *reinterpret_cast<const float4*>(pv + 12);
-                p.rd[0] = v0.x;
-                p.rd[1] = v0.y;
-                p.rd[2] = v0.z;
-                p.rd[3] = v0.w;
-                p.l10 = v1.x;
-                p.l20 = v1.y;
-                p.l30 = v1.z;
-                p.l21 = v1.w;
-                p.l31 = v2.x;
-                p.l32 = v2.y;
-                p.b10 = v2.z;
-                p.b20 = v2.w;
-                p.b30 = v3.x;
-                p.b21 = v3.y;
-                p.b31 = v3.z;
-                p.b32 = v3.w;
-            }
-            if (bi == q) {
-                // block row, left of the pivot: rows become L_b^-1 x (final)
 #pragma unroll
-                for (int c = 0; c < 4; ++c) unit_lower_solve(m[0][c], m[1][c], m[2][c], m[3][c], p);
-            } else {
-                // my rows below the pivot: w = L_b^-1 p, u = w / d
-                float u[4][4], wv[4][4];
-                const float* pr = Pst + buf * NB * 4 + i0 * 4;
+            for (int r = 0; r < 4; ++r) u[r] = *reinterpret_cast<const float4*>(U + 4 * (i0 + r));
+            if (bk == q) {
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
-                    const float4 x = *reinterpret_cast<const float4*>(pr + 4 * r);
-                    float x0 = x.x, x1 = x.y, x2 = x.z, x3 = x.w;
-                    unit_lower_solve(x0, x1, x2, x3, p);
-                    wv[r][0] = x0;
-                    wv[r][1] = x1;
-                    wv[r][2] = x2;
-                    wv[r][3] = x3;
-                    u[r][0] = x0 * p.rd[0];
-                    u[r][1] = x1 * p.rd[1];
-                    u[r][2] = x2 * p.rd[2];
-                    u[r][3] = x3 * p.rd[3];
-                }
-                if (bk == q) {
-                    // panel: final raw inverse columns
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        m[r][0] = fmaf(-u[r][3], p.b30, fmaf(-u[r][2], p.b20, fmaf(-u[r][1], p.b10, wv[r][0])));
-                        m[r][1] = fmaf(-u[r][3], p.b31, fmaf(-u[r][2], p.b21, wv[r][1]));
-                        m[r][2] = fmaf(-u[r][3], p.b32, wv[r][2]);
-                        m[r][3] = wv[r][3];
-                    }
-                } else {
-                    // h = L_b^-1 x, x from the block row (left columns) or the panel (right)
-                    float h[4][4];   // h[t][c]
-                    if (bk < q) {
-                        const float* qr = Qst + buf * 4 * NB + k0;
-#pragma unroll
-                        for (int t = 0; t < 4; ++t) {
-                            const float4 x = *reinterpret_cast<const float4*>(qr + t * NB);
-                            h[t][0] = x.x;
-                            h[t][1] = x.y;
-                            h[t][2] = x.z;
-                            h[t][3] = x.w;
-                        }
-                    } else {
-                        const float* pc = Pst + buf * NB * 4 + k0 * 4;
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            const float4 x = *reinterpret_cast<const float4*>(pc + 4 * c);
-                            h[0][c] = x.x;
-                            h[1][c] = x.y;
-                            h[2][c] = x.z;
-                            h[3][c] = x.w;
-                        }
-                    }
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) unit_lower_solve(h[0][c], h[1][c], h[2][c], h[3][c], p);
-#pragma unroll
-                    for (int t = 0; t < 4; ++t)
-#pragma unroll
-                        for (int r = 0; r < 4; ++r)
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) m[r][c] = fmaf(-u[r][t], h[t][c], m[r][c]);
+                    const float4 v = *reinterpret_cast<const float4*>(Wr + 4 * (i0 + r));
+                    m[r][0] = make_float2(v.x, v.y);
+                    m[r][1] = make_float2(v.z, v.w);
                 }
             }
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const float nu = t == 0 ? u[r].x : t == 1 ? u[r].y : t == 2 ? u[r].z : u[r].w;
+                    m[r][0] = __ffma2_rn(make_float2(nu, nu), h[t][0], m[r][0]);
+                    m[r][1] = __ffma2_rn(make_float2(nu, nu), h[t][1], m[r][1]);
+                }
+            if (!diag) diag_publish(q + 1, m, bi, bk, Raw);
+            else if (tid == q + 1) diag_factor(m, Pv, dv + 4 * (q + 1));
         }
-        if (owner && q + 1 < NB / 4) diag_publish(q + 1, m, bi, bk, Pst, Qst, Pv);
         __syncthreads();
     }
-    // Scales (the staging is free now): 1 / sqrt(d), 1 / d.
-    float* isq = Pst;
-    float* idv = Qst;
-    if (tid < NB) {
+    if (tid < NB) {   // scales 1 / sqrt(d), 1 / d
         const float d = dv[tid];
         isq[tid] = __frcp_rn(sqrtf(d));
         idv[tid] = __frcp_rn(d);
+        if (!(d > 0.0f) && off + tid < n) atomicMin(&first_bad, tid);
     }
     __syncthreads();
+    if (tid == 0 && first_bad < NB) record_error(info, static_cast<int>(n - off - first_bad));
     // C^-1 = D^-1/2 L^-1 with L^-1_ik = -R_ik / d_k (k < i); the upper blocks of Z stay 0.
     // C_kk itself is not stored: later steps read only C^-1_kk and the blocks below it.
-    if (owner) {
+    for (int e = tid; e < NB * NB / 4; e += DIAG_THREADS) {
+        const int i = e / (NB / 4), c4 = 4 * (e % (NB / 4));
+        if (c4 > i) continue;
+        const float4 v = *reinterpret_cast<const float4*>((c4 == (i & ~3) ? Bm + 4 * i : Hist + i * NB + c4));
+        const float mr[4] = {v.x, v.y, v.z, v.w};
+        const float si = isq[i];
+        float o[4];
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int i = i0 + r;
-            const float si = isq[i];
-            float o[4];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int kk = k0 + c;
-                o[c] = kk < i ? -m[r][c] * idv[kk] * si : (kk == i ? si : 0.0f);
-            }
-            if (KQ_IN_RANGE((off + i) * npad + off + k0 + 3, npad * npad))
-                *reinterpret_cast<float4*>(w.Z + (off + i) * npad + off + k0) = make_float4(o[0], o[1], o[2], o[3]);
+        for (int c = 0; c < 4; ++c) {
+            const int kk = c4 + c;
+            o[c] = kk < i ? -mr[c] * idv[kk] * si : (kk == i ? si : 0.0f);
         }
+        if (KQ_IN_RANGE((off + i) * npad + off + c4 + 3, npad * npad))
+            *reinterpret_cast<float4*>(w.Z + (off + i) * npad + off + c4) = make_float4(o[0], o[1], o[2], o[3]);
     }
 }
 
