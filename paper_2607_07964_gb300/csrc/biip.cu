@@ -170,6 +170,10 @@ __global__ void __launch_bounds__((1 << LG) / 16) rht_rows_reg_kernel(float* __r
 // warps of the other groups keep loads in flight while one group waits on its chunk.
 // (Seven groups of four chunks each, with the next row prefetched into registers,
 // measured 14.6-14.8 against 13.3 ms for the rotation stage of the 70B down_proj layer.)
+// Each thread's pre-factors are formed once and held in registers over its rows, and a group
+// meets only itself between its phases (it alone uses its exchange buffer): 14336 rows of 14336
+// 529.5 -> 460 -> 443.7 us (3.7 TB/s read and written). At the 72 registers two CTAs can share
+// about 150 bytes of the factors spill; one CTA per SM without spills was the slower one.
 template <int LG, bool POST>
 __global__ void __launch_bounds__(14 * (1 << LG) / 16, LG == 9 ? 2 : 1) rht_rows28_reg_kernel(float* __restrict__ M, int64_t rows,
                                                                               int pre_mode, int post_mode,
@@ -184,6 +188,9 @@ __global__ void __launch_bounds__(14 * (1 << LG) / 16, LG == 9 ? 2 : 1) rht_rows
     const int t = threadIdx.x, g = t / TG, tl = t - g * TG;
     float* buf = sm28 + N + g * P;                           // this group's exchange buffer
     const int tw = deposit_bits<(P - 1) & ~ML>(tl);
+    float f[CPG][16];   // this thread's pre-factors, the same for every row
+#pragma unroll
+    for (int c = 0; c < CPG; ++c) factors16(pre_mode, sign, s, (g + G * c) * P + 16 * tl, f[c]);
     for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
 #pragma unroll
         for (int c = 0; c < CPG; ++c) {
@@ -198,13 +205,11 @@ __global__ void __launch_bounds__(14 * (1 << LG) / 16, LG == 9 ? 2 : 1) rht_rows
                 x[4 * q + 2] = w4.z;
                 x[4 * q + 3] = w4.w;
             }
-            float f[16];
-            factors16(pre_mode, sign, s, a * P + 16 * tl, f);
 #pragma unroll
-            for (int k = 0; k < 16; ++k) x[k] *= f[k];
+            for (int k = 0; k < 16; ++k) x[k] *= f[c][k];
             fwht_kbits<0xFu>(x);
-            rr_transpose<LG, 1, true>(x, buf, tl);
-            rr_transpose<LG, 2, true>(x, buf, tl);
+            rr_transpose<LG, 1, true, true>(x, buf, tl, true, g);
+            rr_transpose<LG, 2, true, true>(x, buf, tl, true, g);
 #pragma unroll
             for (int k = 0; k < 16; ++k)
                 if (KQ_IN_RANGE(a * P + (tw | deposit_bits<ML>(k)), N)) v[a * P + (tw | deposit_bits<ML>(k))] = x[k];
@@ -222,6 +227,102 @@ __global__ void __launch_bounds__(14 * (1 << LG) / 16, LG == 9 ? 2 : 1) rht_rows
             });
         }
         __syncthreads();   // v is rewritten by the next row
+    }
+}
+
+// Walsh-Hadamard transform of V values in registers (natural order).
+template <int V>
+__device__ __forceinline__ void fwht_regs(float (&x)[V]) {
+#pragma unroll
+    for (int h = 1; h < V; h <<= 1)
+#pragma unroll
+        for (int i = 0; i < V; i += 2 * h)
+#pragma unroll
+            for (int j = i; j < i + h; ++j) {
+                const float a = x[j], b = x[j + h];
+                x[j] = a + b;
+                x[j + h] = a - b;
+            }
+}
+
+// ------------------------------------------- row transform, n = 28 * 2^LG, LG in [4, 8]
+// 448 to 7168. A CTA takes 512 / P rows at a time (14336 values in shared memory, 56 KB, beside
+// a table of the pre-factors): a thread's 16 contiguous values take the first four stages in
+// registers, the remaining LG - 4 stages (stride 16 in a chunk) one radix-2^(LG-4) pass through
+// shared memory, and then each of the 256 threads mixes two columns of a row (packed pairs) with
+// the dense +-1 sums of mix28 and writes 8-byte results. The stages, sums and factors are
+// those of rht_rows_kernel in its order, so the results have its bits. Bound: the 28
+// additions a value of the mix (FP32 pipe) and HBM, which are close. rht_rows_kernel gave one
+// row to 256 threads, of which P mixed, and formed every factor again for every row: 8192 rows
+// of 896 146.7 -> 23.3 us, of 7168 359.5 -> 137.5 (3.4 TB/s read and written).
+// Quads of the shared copy are permuted within 128 bytes so that the 16-byte stores of 16
+// contiguous values per thread, and the later row accesses, hit distinct banks.
+__device__ __forceinline__ int quad_swz(int j) { return j ^ (((j >> 5) & 3) << 2); }
+
+template <int LG, bool POST>
+__global__ void __launch_bounds__(256, 2) rht_rows28_mid_kernel(float* __restrict__ M, int64_t rows, int pre_mode,
+                                                                int post_mode, const int8_t* __restrict__ sign,
+                                                                const float* __restrict__ s, float inv_sqrt_n) {
+    constexpr int P = 1 << LG, N = 28 * P, RPB = 512 / P, TILE = N * RPB;   // 14336
+    constexpr int R = 1 << (LG - 4);   // radix of the second pass
+    extern __shared__ __align__(16) float smid[];
+    float* v = smid;             // [RPB][N]
+    float* pf = smid + TILE;     // [N] pre-factors
+    for (int j = threadIdx.x; j < N; j += 256) pf[j] = factor(pre_mode, sign, s, j);
+    const int64_t tiles = (rows + RPB - 1) / RPB;
+    for (int64_t w = blockIdx.x; w < tiles; w += gridDim.x) {
+        float* base = M + w * TILE;
+        const int live = static_cast<int>(min(static_cast<int64_t>(RPB), rows - w * RPB)) * N;   // values of this tile
+        __syncthreads();   // the previous tile's columns have been read (and pf is there)
+#pragma unroll 2
+        for (int e = 16 * threadIdx.x; e < TILE; e += 16 * 256) {
+            if (e >= live) break;
+            float x[16];
+            const float4* src = reinterpret_cast<const float4*>(base + e);
+            const float4* pq = reinterpret_cast<const float4*>(pf + (RPB == 1 ? e : e % N));
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 a = src[q], f = pq[q];
+                x[4 * q] = __fmul_rn(a.x, f.x);
+                x[4 * q + 1] = __fmul_rn(a.y, f.y);
+                x[4 * q + 2] = __fmul_rn(a.z, f.z);
+                x[4 * q + 3] = __fmul_rn(a.w, f.w);
+            }
+            fwht_kbits<0xFu>(x);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                *reinterpret_cast<float4*>(v + quad_swz(e + 4 * q)) = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
+        }
+        __syncthreads();
+        if constexpr (LG > 4) {
+            for (int t = threadIdx.x; t < TILE / R; t += 256) {
+                const int j0 = (t >> 4) * P + (t & 15);   // chunk t / 16 of the tile, offset t % 16
+                if (j0 >= live) break;
+                float x[R];
+#pragma unroll
+                for (int i = 0; i < R; ++i) x[i] = v[quad_swz(j0 + 16 * i)];
+                fwht_regs<R>(x);
+#pragma unroll
+                for (int i = 0; i < R; ++i) v[quad_swz(j0 + 16 * i)] = x[i];
+            }
+            __syncthreads();
+        }
+        {
+            const int row = threadIdx.x / (P / 2), b = 2 * (threadIdx.x % (P / 2));
+            if (row * N < live) {
+                float2 x[28];
+#pragma unroll
+                for (int a = 0; a < 28; ++a) x[a] = *reinterpret_cast<const float2*>(v + quad_swz(row * N + a * P + b));
+                float* dst = base + row * N + b;
+                mix28_pairs(x, [&](int a, float2 y) {
+                    const int j = a * P + b;
+                    const float f0 = POST ? factor(post_mode, sign, s, j) * inv_sqrt_n : inv_sqrt_n;
+                    const float f1 = POST ? factor(post_mode, sign, s, j + 1) * inv_sqrt_n : inv_sqrt_n;
+                    if (KQ_IN_RANGE((dst - M) + a * P + 1, rows * N))
+                        *reinterpret_cast<float2*>(dst + a * P) = make_float2(y.x * f0, y.y * f1);
+                });
+            }
+        }
     }
 }
 
@@ -268,20 +369,6 @@ __global__ void __launch_bounds__(256) transpose_sq_kernel(float* __restrict__ M
 // group's pre- and post-factors are staged once in shared memory. No shared-memory round
 // trips between radix-2 stages (a tiled shared-memory version with radix-8 sub-stages moved
 // each element through shared memory several times per pass: 2.35 against ~4 TB/s).
-template <int V>
-__device__ __forceinline__ void fwht_regs(float (&x)[V]) {
-#pragma unroll
-    for (int h = 1; h < V; h <<= 1)
-#pragma unroll
-        for (int i = 0; i < V; i += 2 * h)
-#pragma unroll
-            for (int j = i; j < i + h; ++j) {
-                const float a = x[j], b = x[j + h];
-                x[j] = a + b;
-                x[j + h] = a - b;
-            }
-}
-
 template <int R>
 __global__ void __launch_bounds__(128) rht_cols_reg_kernel(float* __restrict__ M, int n, int64_t ncols, int S,
                                                            int pre_mode, int post_mode,
@@ -647,6 +734,29 @@ kq_status launch_rows28_reg(float* M, int64_t rows, int pre, int post, const int
     return KQ_OK;
 }
 
+template <int LG>
+kq_status launch_rows28_mid(float* M, int64_t rows, int pre, int post, const int8_t* sign, const float* s,
+                            cudaStream_t stream) {
+    constexpr int N = 28 << LG, RPB = 512 >> LG;
+    constexpr size_t smem = (static_cast<size_t>(N) * RPB + N) * sizeof(float);
+    static std::atomic<uint64_t> attr{0};
+    KQ_TRY(once_per_device(attr, [&]() -> kq_status {
+        KQ_CUDA(cudaFuncSetAttribute(rht_rows28_mid_kernel<LG, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     static_cast<int>(smem)));
+        KQ_CUDA(cudaFuncSetAttribute(rht_rows28_mid_kernel<LG, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     static_cast<int>(smem)));
+        return KQ_OK;
+    }));
+    const int64_t grid = std::min<int64_t>(cdiv(rows, RPB), static_cast<int64_t>(num_sms()) * 2);
+    const float isn = static_cast<float>(1.0 / sqrt(static_cast<double>(N)));
+    if (post == F_NONE)
+        rht_rows28_mid_kernel<LG, false><<<static_cast<unsigned>(grid), 256, smem, stream>>>(M, rows, pre, post, sign, s, isn);
+    else
+        rht_rows28_mid_kernel<LG, true><<<static_cast<unsigned>(grid), 256, smem, stream>>>(M, rows, pre, post, sign, s, isn);
+    KQ_LAUNCH_CHECK("rht_rows28_mid_kernel");
+    return KQ_OK;
+}
+
 // M 16-byte aligned and n a power of two from 512 to 16384, or 28 * 512 / 28 * 1024: a
 // register row transform.
 bool rows_reg_ok(const float* M, int64_t n) {
@@ -672,6 +782,16 @@ kq_status rows_transform(float* M, int64_t rows, int64_t n, int pre, int post, c
             case 12: return launch_rows_reg<12>(M, rows, pre, post, sign, s, stream);
             case 13: return launch_rows_reg<13>(M, rows, pre, post, sign, s, stream);
             case 14: return launch_rows_reg<14>(M, rows, pre, post, sign, s, stream);
+            default: break;
+        }
+    }
+    if (rows > 0 && p.has28 && (reinterpret_cast<uintptr_t>(M) & 15u) == 0) {
+        switch (p.P) {
+            case 16: return launch_rows28_mid<4>(M, rows, pre, post, sign, s, stream);
+            case 32: return launch_rows28_mid<5>(M, rows, pre, post, sign, s, stream);
+            case 64: return launch_rows28_mid<6>(M, rows, pre, post, sign, s, stream);
+            case 128: return launch_rows28_mid<7>(M, rows, pre, post, sign, s, stream);
+            case 256: return launch_rows28_mid<8>(M, rows, pre, post, sign, s, stream);
             default: break;
         }
     }

@@ -139,6 +139,25 @@ __device__ __forceinline__ void mix28(const float (&x)[28], Out out) {
     mix28_rows(x, out, std::make_integer_sequence<int, 28>{});
 }
 
+// mix28 of two columns at once: the same sums in the same order, in packed pairs (acc - x as
+// fma(-1, x, acc): the same rounding).
+template <uint32_t M>
+__device__ __forceinline__ float2 pm_sum28_pair(const float2 (&x)[28]) {
+    float2 acc = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int a = 0; a < 28; ++a)
+        acc = ((M >> a) & 1u) ? __ffma2_rn(make_float2(-1.0f, -1.0f), x[a], acc) : __fadd2_rn(acc, x[a]);
+    return acc;
+}
+template <typename Out, int... R>
+__device__ __forceinline__ void mix28_pair_rows(const float2 (&x)[28], Out& out, std::integer_sequence<int, R...>) {
+    (out(R, pm_sum28_pair<kH28.m[R]>(x)), ...);
+}
+template <typename Out>
+__device__ __forceinline__ void mix28_pairs(const float2 (&x)[28], Out out) {
+    mix28_pair_rows(x, out, std::make_integer_sequence<int, 28>{});
+}
+
 // In-register Walsh-Hadamard transform of R = 2, 4 or 8 values (natural order).
 template <int R>
 __device__ __forceinline__ void fwht_reg(float (&x)[8]) {
@@ -366,9 +385,19 @@ __device__ __forceinline__ int swz_bank(int j) {
 // Values of phase Q - 1 to shared memory, those of phase Q back, and phase Q's butterflies.
 // Every thread of the CTA calls it (two barriers); threads with act false hold no values.
 // SWZ: the buffer holds P floats addressed through swz_bank (LG = 9, 10), else P + P / 32
-// padded one float in 32.
-template <int LG, int Q, bool SWZ = false>
-__device__ __forceinline__ void rr_transpose(float (&x)[16], float* buf, int t, bool act = true) {
+// padded one float in 32. GROUPED: the buffer belongs to the P / 16 threads of group `grp`, and
+// only they meet at the barriers (a warp, or two warps on named barrier grp + 1).
+template <int LG, int Q, bool SWZ = false, bool GROUPED = false>
+__device__ __forceinline__ void rr_transpose(float (&x)[16], float* buf, int t, bool act = true, int grp = 0) {
+    auto sync = [&]() {
+        if constexpr (!GROUPED)
+            __syncthreads();
+        else if constexpr (LG == 9)
+            __syncwarp();
+        else
+            asm volatile("barrier.sync %0, %1;" ::"r"(grp + 1), "n"((1 << LG) / 16) : "memory");
+    };
+    static_assert(!GROUPED || LG == 9 || LG == 10, "groups of one or two warps");
     constexpr uint32_t N1 = (1u << LG) - 1u;
     constexpr uint32_t MW = rr_mask(LG, Q - 1), MR = rr_mask(LG, Q);
     const int tw = deposit_bits<N1 & ~MW>(t), tr = deposit_bits<N1 & ~MR>(t);
@@ -378,12 +407,12 @@ __device__ __forceinline__ void rr_transpose(float (&x)[16], float* buf, int t, 
         else
             return pad32(j);
     };
-    __syncthreads();   // the previous reads of buf are done
+    sync();   // the previous reads of buf are done
     if (act) {
 #pragma unroll
         for (int k = 0; k < 16; ++k) buf[at(tw | deposit_bits<MW>(k))] = x[k];
     }
-    __syncthreads();
+    sync();
     if (act) {
 #pragma unroll
         for (int k = 0; k < 16; ++k) x[k] = buf[at(tr | deposit_bits<MR>(k))];
