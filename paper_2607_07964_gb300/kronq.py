@@ -103,17 +103,20 @@ def _ok(st: int, where: str) -> None:
         raise KronqError(st, where, last_error())
 
 
+# Pointers and the stream as plain integers: the declared argument types convert them.
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    return (torch.cuda.current_stream() if stream is None else stream).cuda_stream
 
 
 def _need(t, name, dtype, shape=None, contiguous=True):
     if t is None:
+        return
+    # one test for what is nearly always so; the errors are sorted out below
+    if t.is_cuda and t.dtype is dtype and (shape is None or t.shape == shape) and (not contiguous or t.is_contiguous()):
         return
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")

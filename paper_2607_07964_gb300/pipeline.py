@@ -131,7 +131,7 @@ class LayerPipeline:
         for c, (t0, t1) in enumerate(ch):
             if ready is not None:
                 stream.wait_event(ready[c])
-            kq.kq_accum_factor(A[t0:t1], H, accumulate=c > 0, trace=trace if c == len(ch) - 1 else None,
+            kq.kq_accum_factor(A if len(ch) == 1 else A[t0:t1], H, accumulate=c > 0, trace=trace if c == len(ch) - 1 else None,
                                info=info, stream=stream)
 
     def _need_xt(self, Xt) -> None:
