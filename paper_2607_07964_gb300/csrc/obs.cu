@@ -17,8 +17,8 @@
 //             acc = fma(-wpre_k, P_kc, acc) over ascending k; w_c = w_c - acc
 // Kernels:
 //   rowgrid_kernel   per-row grid (group = 0) from the whole row before the sweep
-//   pack_r_kernel    the diagonal 128 x 128 blocks of R as the block kernel's 16 x 16 tiles
-//   pack_rq_kernel   the blocks of R right of them, for the fused update
+//   pack_r_kernel    the diagonal 128 x 128 blocks of R as the block kernel's 16 x 16 tiles, and
+//                    the blocks of R right of them, for the fused update
 //   obs_block_kernel 32 rows per CTA, lane = row, 16 columns per warp
 //   trailing_kernel  128 x 128 output tiles of the shared tile GEMM (tile_gemm.cuh)
 //   colloss_kernel   col_loss[j] = sum over rows of E_j^2, fixed order (sumsq.cuh)
@@ -132,21 +132,22 @@ static_assert(OBS_ROWS * PLD <= NWARP * XT, "E_prev is staged in the exchange ti
 enum { FUSE_NONE = 0, FUSE_FP32 = 1, FUSE_MMA = 2 };
 
 // Rp[b][tile(o, s)][jj][t] = R[i0 + 16 o + jj][i0 + 16 s + t] = Lt[i0 + 16 s + t][i0 + 16 o + jj]
-// (0 outside the matrix; diagonal tiles shifted as above), i0 = b BLK. Grid (RTILES, blocks), block (16, 16): one tile.
-__global__ void pack_r_kernel(const float* __restrict__ Lt, int64_t n, float* __restrict__ Rp) {
+// (0 outside the matrix; diagonal tiles shifted as above), i0 = b BLK, b = blockIdx.y: tile `tile` by 256 threads.
+__device__ __forceinline__ void pack_r_tile(const float* __restrict__ Lt, int64_t n, float* __restrict__ Rp, int tile) {
     __shared__ float t[CW][CW + 1];
-    int s = 0, o = static_cast<int>(blockIdx.x);
+    const int tx = threadIdx.x % CW, ty = threadIdx.x / CW;
+    int s = 0, o = tile;
     while (o > s) {
         o -= s + 1;
         ++s;
     }
     const int64_t i0 = static_cast<int64_t>(blockIdx.y) * BLK;
-    const int64_t c = i0 + CW * s + threadIdx.y, j = i0 + CW * o + threadIdx.x;
-    t[threadIdx.y][threadIdx.x] = (c < n && j < n) ? Lt[c * n + j] : 0.0f;
+    const int64_t c = i0 + CW * s + ty, j = i0 + CW * o + tx;
+    t[ty][tx] = (c < n && j < n) ? Lt[c * n + j] : 0.0f;
     __syncthreads();
-    const int64_t e = static_cast<int64_t>(blockIdx.y) * RPACK + rtile(o, s) + threadIdx.y * CW + threadIdx.x;
-    const int jj = threadIdx.y;
-    int tt = threadIdx.x;   // column within the tile
+    const int64_t e = static_cast<int64_t>(blockIdx.y) * RPACK + rtile(o, s) + ty * CW + tx;
+    const int jj = ty;
+    int tt = tx;   // column within the tile
     if (o == s) tt += PUB * (jj / PUB);
     if (KQ_IN_RANGE(e, static_cast<int64_t>(gridDim.y) * RPACK)) Rp[e] = tt < CW ? t[tt][jj] : 0.0f;
 }
@@ -156,10 +157,9 @@ __global__ void pack_r_kernel(const float* __restrict__ Lt, int64_t n, float* __
 // of 16 columns as four uniform 16-byte loads. FRAG = true: Rq[b][s][ks][lane][4] =
 // (R[8 ks + t4][c], R[8 ks + t4 + 4][c], the same at c + 8), c = 16 s + g, g = lane / 4,
 // t4 = lane % 4: the B fragments of mma.sync m16n8k8 for warp s's two column tiles, one
-// 16-byte load per lane and k step. Grid (8, blocks), block 256.
+// 16-byte load per lane and k step. b = blockIdx.y; warp s's part by 256 threads.
 template <bool FRAG>
-__global__ void pack_rq_kernel(const float* __restrict__ Lt, int64_t n, float* __restrict__ Rq) {
-    const int s = static_cast<int>(blockIdx.x);
+__device__ __forceinline__ void pack_rq_part(const float* __restrict__ Lt, int64_t n, float* __restrict__ Rq, int s) {
     const int64_t i0 = static_cast<int64_t>(blockIdx.y) * BLK, i1 = i0 + BLK + CW * s;
     float* out = Rq + static_cast<int64_t>(blockIdx.y) * BLK * BLK + s * BLK * CW;
     __shared__ float t[CW][BLK + 1];
@@ -177,6 +177,20 @@ __global__ void pack_rq_kernel(const float* __restrict__ Lt, int64_t n, float* _
             v = t[e % CW][e / CW];
         }
         if (KQ_IN_RANGE(e, CW * BLK)) out[e] = v;
+    }
+}
+
+// Both packings in one launch: a launch costs a short sweep as much as the copying does.
+// Grid (RTILES, blocks), or with RQ != PACK_NONE (RTILES + NWARP, blocks); block 256.
+enum { PACK_NONE = 0, PACK_ROWS = 1, PACK_FRAG = 2 };
+template <int RQ>
+__global__ void __launch_bounds__(256) pack_r_kernel(const float* __restrict__ Lt, int64_t n, float* __restrict__ Rp,
+                                                     float* __restrict__ Rq) {
+    const int x = static_cast<int>(blockIdx.x);
+    if (x < RTILES) {
+        pack_r_tile(Lt, n, Rp, x);
+    } else if constexpr (RQ != PACK_NONE) {
+        if (blockIdx.y + 1 < gridDim.y) pack_rq_part<RQ == PACK_FRAG>(Lt, n, Rq, x - RTILES);   // the last block has no next
     }
 }
 
@@ -339,7 +353,7 @@ __device__ __forceinline__ void column_step(float w, const RowGrid& g, float2 d,
 // and codes move as 16-byte vectors. HASP: with the GPTAQ correction; Pp is P's
 // diagonal block packed like R's, and the block's -Wpre goes to Q (fp32 trailing update)
 // or to Qh + Ql (tensor-core trailing update). FUSE: the previous block's update of this
-// block column first (Rq: pack_rq_kernel's layout for that form). One CTA per 32 rows.
+// block column first (Rq: pack_rq_part's layout for that form). One CTA per 32 rows.
 template <bool VEC, bool HASP, int FUSE, int PER_SM = 2>
 __global__ void __launch_bounds__(OBS_THREADS, PER_SM) obs_block_kernel(
     const float* W, int64_t d_out, int64_t d_in, const float* __restrict__ Rp, int64_t i0,
@@ -869,16 +883,6 @@ extern "C" kq_status kq_obs_quantize(float* W, int64_t d_out, int64_t d_in, cons
     }));
     ObsWs o = carve(ws, d_out, d_in, mode, hp);
     TrailMaps maps;
-    if (tc) {
-        kq_status st0 = split_tf32(Lt, d_in * d_in, o.Lh, o.Ll, stream);
-        if (st0 != KQ_OK) return st0;
-        if ((st0 = maps.init(o.Eh, o.El, o.Lh, o.Ll, d_out, d_in)) != KQ_OK) return st0;
-        if ((st0 = maps.set_w(W, d_out, d_in)) != KQ_OK) return st0;
-        if (hp) {
-            if ((st0 = split_tf32(Pt, d_in * d_in, o.Ph, o.Pl, stream)) != KQ_OK) return st0;
-            if ((st0 = maps.init_p(o.Qh, o.Ql, o.Ph, o.Pl, d_out, d_in)) != KQ_OK) return st0;
-        }
-    }
     if (group == 0) {
         rowgrid_kernel<<<static_cast<unsigned>(cdiv(d_out, 8)), 256, 0, stream>>>(W, d_out, d_in, bits, scale,
                                                                                 zero, o.gscale, o.gzero);
@@ -889,23 +893,34 @@ extern "C" kq_status kq_obs_quantize(float* W, int64_t d_out, int64_t d_in, cons
                       (reinterpret_cast<uintptr_t>(codes) % 16 == 0);
     const int64_t nblk = cdiv(d_in, BLK);
     const int64_t row_ctas = cdiv(d_out, OBS_ROWS);
-    pack_r_kernel<<<dim3(RTILES, static_cast<unsigned>(nblk)), dim3(CW, CW), 0, stream>>>(Lt, d_in, o.Rp);
-    KQ_LAUNCH_CHECK("pack_r_kernel");
     // the blocks of R right of the diagonal ones, for the fused update: as mma.sync fragments in
     // the 3xTF32 mode, as rows otherwise
     const bool fuse_ok = !hp && nblk > 1 && row_ctas <= static_cast<int64_t>(num_sms()) &&
                          d_out * d_in <= (int64_t{24} << 20);
     const bool mma_fused = fuse_ok && tc && bvec;
-    if (fuse_ok) {
-        const dim3 rqgrid(NWARP, static_cast<unsigned>(nblk - 1));
+    {
+        const dim3 pgrid(RTILES + (fuse_ok ? NWARP : 0), static_cast<unsigned>(nblk));
         if (mma_fused)
-            pack_rq_kernel<true><<<rqgrid, 256, 0, stream>>>(Lt, d_in, o.Rq);
+            pack_r_kernel<PACK_FRAG><<<pgrid, 256, 0, stream>>>(Lt, d_in, o.Rp, o.Rq);
+        else if (fuse_ok)
+            pack_r_kernel<PACK_ROWS><<<pgrid, 256, 0, stream>>>(Lt, d_in, o.Rp, o.Rq);
         else
-            pack_rq_kernel<false><<<rqgrid, 256, 0, stream>>>(Lt, d_in, o.Rq);
-        KQ_LAUNCH_CHECK("pack_rq_kernel");
+            pack_r_kernel<PACK_NONE><<<pgrid, 256, 0, stream>>>(Lt, d_in, o.Rp, nullptr);
+        KQ_LAUNCH_CHECK("pack_r_kernel");
+    }
+    // L split for the trailing updates, unless there are none: one block, or two with the fused update
+    if (tc && nblk > (fuse_ok ? 2 : 1)) {
+        kq_status st0 = split_tf32(Lt, d_in * d_in, o.Lh, o.Ll, stream);
+        if (st0 != KQ_OK) return st0;
+        if ((st0 = maps.init(o.Eh, o.El, o.Lh, o.Ll, d_out, d_in)) != KQ_OK) return st0;
+        if ((st0 = maps.set_w(W, d_out, d_in)) != KQ_OK) return st0;
+        if (hp) {
+            if ((st0 = split_tf32(Pt, d_in * d_in, o.Ph, o.Pl, stream)) != KQ_OK) return st0;
+            if ((st0 = maps.init_p(o.Qh, o.Ql, o.Ph, o.Pl, d_out, d_in)) != KQ_OK) return st0;
+        }
     }
     if (hp) {   // P[i0 + j][i0 + c] = Pt[i0 + c][i0 + j]: the same packing as R from Lt
-        pack_r_kernel<<<dim3(RTILES, static_cast<unsigned>(nblk)), dim3(CW, CW), 0, stream>>>(Pt, d_in, o.Pp);
+        pack_r_kernel<PACK_NONE><<<dim3(RTILES, static_cast<unsigned>(nblk)), 256, 0, stream>>>(Pt, d_in, o.Pp, nullptr);
         KQ_LAUNCH_CHECK("pack_r_kernel");
     }
     // GPTQ mode: block b's kernel first applies the previous block's update of its own
