@@ -14,8 +14,8 @@
 // where B (stored in Z's blocks) is the right-hand side I of C Z = I after the earlier
 // steps' eliminations. The matrix is padded to a multiple of nb with an identity block.
 // Look-ahead: the update is split into the tiles step k + 1 reads first (row and column
-// block k + 1; the next diagonal tile alone on the caller's stream, the rest on a library
-// side stream) and the rest of the step's tiles (side stream, beside step k + 1's diagonal
+// block k + 1; the next diagonal tile alone on the caller's stream, by the panel kernel itself
+// or after it, the rest on a library side stream) and the rest of the step's tiles (side stream, beside step k + 1's diagonal
 // factorization and panel). The diagonal kernel is fp32 SIMT with fused multiply-add; the
 // panel and the tile updates multiply on the tensor cores (mma.sync tf32 with the 3xTF32
 // split, operands split as they are loaded).
@@ -271,6 +271,7 @@ __global__ void __launch_bounds__(DIAG_THREADS) chol_diag_kernel(Work w, int64_t
     const bool owner = bi < NB / 4;   // the last 16 threads own nothing
     const int i0 = 4 * bi, k0 = 4 * bk;
     float2 m[4][2] = {};
+    pdl_wait();   // the kernel that updated this tile
     if (owner) {
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
@@ -484,33 +485,6 @@ __device__ __forceinline__ void strip_gemm(const float* __restrict__ A, const fl
         for (int j = 0; j < CN; ++j) acc[i][j] = Cs[(ty + 16 * i) * CLD + (BNL ? CN * tx + j : tx + 16 * j)];
 }
 
-__global__ void __launch_bounds__(G_THREADS, 2) chol_panel_kernel(Work w, int64_t npad, int k, int b0) {
-    extern __shared__ __align__(16) float sm[];
-    const int b = static_cast<int>(blockIdx.x) + b0, s = blockIdx.y;
-    const int64_t off = static_cast<int64_t>(k) * NB;
-    const float* cinv = w.Z + off * npad + off;
-    const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-    if (b < k) {
-        float* out = w.Z + off * npad + static_cast<int64_t>(b) * NB + 32 * s;
-        float acc[8][2];
-        strip_gemm<128, 32, true>(cinv, out, npad, acc, sm);
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-            if (KQ_IN_RANGE((out - w.Z) + (ty + 16 * i) * npad + 2 * tx + 1, npad * npad))
-                *reinterpret_cast<float2*>(out + (ty + 16 * i) * npad + 2 * tx) = make_float2(acc[i][0], acc[i][1]);
-    } else {
-        float* out = w.A + (static_cast<int64_t>(b + 1) * NB + 32 * s) * npad + off;
-        float acc[2][8];
-        strip_gemm<32, 128, false>(out, cinv, npad, acc, sm);
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (KQ_IN_RANGE((out - w.A) + (ty + 16 * i) * npad + tx + 16 * j, npad * npad))
-                    out[(ty + 16 * i) * npad + tx + 16 * j] = acc[i][j];
-    }
-}
-
 // Quadrant q (rows 64 (q / 2), columns 64 (q % 2)) of update tile (i, j) of step k.
 __device__ __forceinline__ void update_quad(const Work& w, int64_t npad, int k, int i, int j, int q, float* sm) {
     const int64_t ko = static_cast<int64_t>(k) * NB;
@@ -547,6 +521,44 @@ __device__ __forceinline__ void update_quad(const Work& w, int64_t npad, int k, 
     }
 }
 
+// The panel of step k: block row index b (b < k: Z_kb, else C_{b+1,k}) in four strips of 32 rows
+// or columns, one CTA each. next: the four CTAs of C_{k+1,k} are a cluster and go on to the update
+// of the diagonal tile (k + 1, k + 1), a quadrant each: a launch less in the chain from one
+// diagonal step to the next, which is bound by launches and latencies (n = 1024: 374 -> 321 us,
+// 40 us a step, of which the diagonal kernel takes 25; with the diagonal step launched as a
+// programmatic dependent alone 348).
+__global__ void __launch_bounds__(G_THREADS, 2) chol_panel_kernel(Work w, int64_t npad, int k, int b0, int next) {
+    extern __shared__ __align__(16) float sm[];
+    const int b = static_cast<int>(blockIdx.y) + b0, s = blockIdx.x;
+    pdl_launch_dependents();   // the next diagonal step: it waits for this grid's end itself
+    const int64_t off = static_cast<int64_t>(k) * NB;
+    const float* cinv = w.Z + off * npad + off;
+    const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+    if (b < k) {
+        float* out = w.Z + off * npad + static_cast<int64_t>(b) * NB + 32 * s;
+        float acc[8][2];
+        strip_gemm<128, 32, true>(cinv, out, npad, acc, sm);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (KQ_IN_RANGE((out - w.Z) + (ty + 16 * i) * npad + 2 * tx + 1, npad * npad))
+                *reinterpret_cast<float2*>(out + (ty + 16 * i) * npad + 2 * tx) = make_float2(acc[i][0], acc[i][1]);
+    } else {
+        float* out = w.A + (static_cast<int64_t>(b + 1) * NB + 32 * s) * npad + off;
+        float acc[2][8];
+        strip_gemm<32, 128, false>(out, cinv, npad, acc, sm);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (KQ_IN_RANGE((out - w.A) + (ty + 16 * i) * npad + tx + 16 * j, npad * npad))
+                    out[(ty + 16 * i) * npad + tx + 16 * j] = acc[i][j];
+    }
+    if (next && b == k) {   // (the four CTAs of a cluster share b) row block k + 1 is complete
+        cluster_barrier();
+        update_quad(w, npad, k, k + 1, k + 1, s, sm);
+    }
+}
+
 // The tiles that step k + 1 reads first: row block k + 1 (tiles (k + 1, j), b0 <= j <= k + 1)
 // and block column k + 1 below it (tiles (i, k + 1), k + 1 < i < b0 + gridDim.x); one tile
 // x 4 quadrants per block index from b0. part 0: all of them; part 1: only the diagonal
@@ -554,6 +566,7 @@ __device__ __forceinline__ void update_quad(const Work& w, int64_t npad, int k, 
 // but that tile, for the next panel.
 __global__ void __launch_bounds__(G_THREADS, 2) chol_next_kernel(Work w, int64_t npad, int k, int part, int b0) {
     extern __shared__ __align__(16) float sm[];
+    pdl_launch_dependents();   // part 1: the next diagonal step (it waits for this grid's end itself)
     const int bid = part == 1 ? k + 1 : static_cast<int>(blockIdx.x) + b0;
     if (part == 2 && bid == k + 1) return;
     if (bid < k + 2)
@@ -750,6 +763,11 @@ extern "C" size_t kq_chol_inv_workspace(int64_t n) {
     return ws_bytes_for(npad_of(n));
 }
 
+// Up to this many blocks the panel kernel also updates the next diagonal tile (chol_panel_kernel).
+// Its clusters of four wait for four free SMs of one GPC, which the far updates of a larger
+// matrix seldom leave: n = 1024 348 -> 321 us, 4096 1734 -> 1624, 5120 2215 -> 2075, but 8192
+// 4054 -> 4234, 14336 10213 -> 10570 (a captured graph: 6144 2456 -> 2537).
+constexpr int NEXT_MAX = 40;
 extern "C" kq_status kq_chol_inv(const float* H, int64_t n, float damp_rel, float* Lt, int* info, void* ws,
                                  size_t ws_bytes, kq_stream_t stream_) {
     cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
@@ -806,6 +824,7 @@ extern "C" kq_status kq_chol_inv(const float* H, int64_t n, float damp_rel, floa
     bool forked = false, remote_pending = false;
     bool next_pending = false;   // the next panel's tiles, updated on the side stream
     const int free_sms = far_free_sms();
+    const bool next_in_panel = side && nbk <= NEXT_MAX;
     for (int k0 = 0; k0 < nbk; k0 += (two_level ? SPB : nbk)) {
         const int k1 = two_level ? std::min(nbk, k0 + SPB) : nbk;   // this super-panel: blocks [k0, k1)
         const int set = two_level ? (k0 / SPB) & 1 : 0;
@@ -813,34 +832,48 @@ extern "C" kq_status kq_chol_inv(const float* H, int64_t n, float damp_rel, floa
         // The steps of the super-panel inside its own blocks: A's lower tiles in rows and
         // columns [k0, k1) and B's tiles in rows and columns [k0, k1).
         for (int k = k0; k < k1; ++k) {
-            chol_diag_kernel<<<1, DIAG_THREADS, DIAG_SMEM, stream>>>(w, n, npad, k, info);
+            // (inside the super-panel the kernel before it on this stream is the one that updated its tile)
+            KQ_CUDA(launch_dependent(chol_diag_kernel, dim3(1), dim3(DIAG_THREADS), DIAG_SMEM, stream, 1u, k > k0, w, n, npad,
+                                     k, info));
             KQ_LAUNCH_CHECK("chol_diag_kernel");
             if (next_pending) {   // the tiles of this panel, updated beside the diagonal step
                 KQ_CUDA(cudaStreamWaitEvent(stream, side->ev2[2], 0));
                 next_pending = false;
             }
+            const bool has_next = k + 1 < k1, in_panel = has_next && next_in_panel;
+            auto rest_done = [&]() -> kq_status {   // the rest of step k - 1 wrote the next diagonal tile
+                if (forked) KQ_CUDA(cudaStreamWaitEvent(stream, side->ev[1], 0));
+                forked = false;
+                return KQ_OK;
+            };
+            if (in_panel) KQ_TRY(rest_done());
             if (k1 - 1 - k0 > 0) {
-                chol_panel_kernel<<<dim3(k1 - 1 - k0, 4), G_THREADS, STRIP_SMEM, stream>>>(w, npad, k, k0);
+                KQ_CUDA(launch_dependent(chol_panel_kernel, dim3(4, static_cast<unsigned>(k1 - 1 - k0)), dim3(G_THREADS), STRIP_SMEM,
+                                         stream, in_panel ? 4u : 1u, false, w, npad, k, k0, in_panel ? 1 : 0));
                 KQ_LAUNCH_CHECK("chol_panel_kernel");
             }
-            if (k + 1 >= k1) break;
+            if (!has_next) break;
             const bool has_rest = k + 2 < k1;   // tiles of this super-panel beyond k + 1
-            if (side) KQ_CUDA(cudaEventRecord(side->ev[0], stream));       // panel k done
-            if (forked) KQ_CUDA(cudaStreamWaitEvent(stream, side->ev[1], 0));   // rest of step k - 1 done
             if (side) {
-                // Step k's update of the next diagonal tile alone on this stream, so the next
-                // diagonal step starts at once; the other tiles the next panel reads, then the
-                // rest of the step's update (other tiles), on the side stream beside it.
+                // Step k's update of the next diagonal tile alone on this stream (by the panel
+                // kernel or its own), so the next diagonal step starts at once; the other tiles
+                // the next panel reads, then the rest of the step's update (other tiles), on the
+                // side stream beside it.
+                KQ_CUDA(cudaEventRecord(side->ev[0], stream));       // panel k done
+                if (!in_panel) KQ_TRY(rest_done());
                 KQ_CUDA(cudaStreamWaitEvent(side->s, side->ev[0], 0));
                 chol_next_kernel<<<dim3(k1 - k0, 4), G_THREADS, STRIP_SMEM, side->s>>>(w, npad, k, 2, k0);
                 KQ_LAUNCH_CHECK("chol_next_kernel");
                 KQ_CUDA(cudaEventRecord(side->ev2[2], side->s));
                 next_pending = true;
-                chol_next_kernel<<<dim3(1, 4), G_THREADS, STRIP_SMEM, stream>>>(w, npad, k, 1, k0);
+                if (!in_panel) {
+                    chol_next_kernel<<<dim3(1, 4), G_THREADS, STRIP_SMEM, stream>>>(w, npad, k, 1, k0);
+                    KQ_LAUNCH_CHECK("chol_next_kernel");
+                }
             } else {
                 chol_next_kernel<<<dim3(k1 - k0, 4), G_THREADS, STRIP_SMEM, stream>>>(w, npad, k, 0, k0);
+                KQ_LAUNCH_CHECK("chol_next_kernel");
             }
-            KQ_LAUNCH_CHECK("chol_next_kernel");
             if (has_rest) {
                 const int m = k1 - k - 2;
                 const unsigned tiles = static_cast<unsigned>(m * (m + 1) / 2 + m * (k - k0 + 1));
