@@ -110,7 +110,7 @@ __device__ __forceinline__ void st_cluster_f4(uint32_t addr, float4 v) {
 template <bool CROSS, int KS>
 __device__ __forceinline__ void gram_tc_body(const CUtensorMap* a0, const CUtensorMap* a1,
                                              const CUtensorMap* bmap, float* __restrict__ H, int d,
-                                             int T, int n_row_tiles, int chunk_stages, int accumulate,
+                                             int T, int n_row_tiles, int tile0, int chunk_stages, int accumulate,
                                              int* info) {
     constexpr int STAGES = stages_of(KS);
     extern __shared__ uint8_t smem_raw[];
@@ -129,7 +129,7 @@ __device__ __forceinline__ void gram_tc_body(const CUtensorMap* a0, const CUtens
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const int tile = static_cast<int>(blockIdx.x) / KS;
+    const int tile = tile0 + static_cast<int>(blockIdx.x) / KS;
     const int rank = KS > 1 ? static_cast<int>(cluster_ctarank()) : 0;
     int ti, tj;
     if (CROSS) {
@@ -474,8 +474,8 @@ __device__ __forceinline__ void gram_tc_body(const CUtensorMap* a0, const CUtens
 template <int KS>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 syrk_tc_kernel(const __grid_constant__ CUtensorMap tmap, float* __restrict__ H, int d, int T,
-               int n_row_tiles, int chunk_stages, int accumulate, int* info) {
-    gram_tc_body<false, KS>(&tmap, &tmap, &tmap, H, d, T, n_row_tiles, chunk_stages, accumulate, info);
+               int n_row_tiles, int tile0, int chunk_stages, int accumulate, int* info) {
+    gram_tc_body<false, KS>(&tmap, &tmap, &tmap, H, d, T, n_row_tiles, tile0, chunk_stages, accumulate, info);
 }
 
 template <int KS>
@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 drift_tc_kernel(const __grid_constant__ CUtensorMap a_hi, const __grid_constant__ CUtensorMap a_lo,
                 const __grid_constant__ CUtensorMap b, float* __restrict__ D, int d, int T,
                 int n_row_tiles, int chunk_stages, int accumulate, int* info) {
-    gram_tc_body<true, KS>(&a_hi, &a_lo, &b, D, d, T, n_row_tiles, chunk_stages, accumulate, info);
+    gram_tc_body<true, KS>(&a_hi, &a_lo, &b, D, d, T, n_row_tiles, 0, chunk_stages, accumulate, info);
 }
 
 // CTAs that share a tile: four while all of them still run at once (one per SM) and each has a chunk.
@@ -610,6 +610,12 @@ KQ_DEBUG_UNIT(syrk)
 extern "C" kq_status kq_accum_factor(const uint16_t* A, int64_t T, int64_t d, int64_t lda,
                                      float* H, int accumulate, double* trace, int* info,
                                      kq_stream_t stream_) {
+    return kq_accum_factor_beside(A, T, d, lda, H, accumulate, trace, info, 0, stream_);
+}
+
+extern "C" kq_status kq_accum_factor_beside(const uint16_t* A, int64_t T, int64_t d, int64_t lda,
+                                            float* H, int accumulate, double* trace, int* info,
+                                            int beside, kq_stream_t stream_) {
     using namespace kq;
     cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
     if (!H || d < 1 || d > 65536 || T < 0 || (T > 0 && !A) || lda < d) {
@@ -638,11 +644,22 @@ extern "C" kq_status kq_accum_factor(const uint16_t* A, int64_t T, int64_t d, in
         int64_t tiles = 0;
         for (int j = 0; j < n_col; ++j) tiles += (n_row - 2 * j > 0) ? n_row - 2 * j : 0;
         const int ks = ks_of(tiles, cdiv(T, KQ_SYRK_CHUNK_TOKENS));
+        // Beside other work: a launch per wave, of equally many tiles, so that the SMs the last wave
+        // would leave idle are free all the time (272 tiles on 152 SMs: twice 136; the inverse
+        // Cholesky's chain beside them does not wait a tile's whole sum for an SM). Layers, us:
+        // 4096 x 4096 and 131072 tokens 5743 -> 5528, 7168 x 4096 and 65536 6396 -> 6095; 16384 tokens
+        // 3419 -> 3432 (a tile takes 0.1 ms there) and 262144 8298 -> 8423 (a wave's tiles end up to
+        // 0.1 ms apart), hence the range. Fewer tiles at a time (91, three waves) 5676, 68 6438.
+        const int64_t waves = beside && ks == 1 && T >= 32768 && T < 196608 ? cdiv(tiles, num_sms()) : 1;
+        const int64_t per = cdiv(tiles, waves);   // tiles per launch
         auto go = [&](auto* kern) -> kq_status {
-            KQ_CUDA(launch_dependent(kern, dim3(static_cast<unsigned>(tiles * ks)), dim3(NUM_THREADS), smem_bytes(ks), stream,
-                                     static_cast<unsigned>(ks), false, tmap, H, static_cast<int>(d), static_cast<int>(T),
-                                     n_row, syrk_chunk_stages(), accumulate, info));
-            KQ_LAUNCH_CHECK("syrk_tc_kernel");
+            for (int64_t t0 = 0; t0 < tiles; t0 += per) {
+                const int64_t nt = std::min(per, tiles - t0);
+                KQ_CUDA(launch_dependent(kern, dim3(static_cast<unsigned>(nt * ks)), dim3(NUM_THREADS), smem_bytes(ks), stream,
+                                         static_cast<unsigned>(ks), false, tmap, H, static_cast<int>(d), static_cast<int>(T),
+                                         n_row, static_cast<int>(t0), syrk_chunk_stages(), accumulate, info));
+                KQ_LAUNCH_CHECK("syrk_tc_kernel");
+            }
             return KQ_OK;
         };
         KQ_TRY(ks == 4 ? go(syrk_tc_kernel<4>) : go(syrk_tc_kernel<1>));

@@ -53,6 +53,7 @@ def lib() -> ctypes.CDLL:
             "kq_debug_status": ([P, P, I], I),
             "kq_selftest_bounds": ([P, I64, P], I),
             "kq_selftest_div": ([P, P, I64, P, P], I),
+            "kq_accum_factor_beside": ([P, I64, I64, I64, P, I, P, P, I, P], I),
             "kq_accum_factor": ([P, I64, I64, I64, P, I, P, P, P], I),
             "kq_compute_scales": ([P, I64, I64, P, P, P, P, P], I),
             "kq_compute_scales_diag": ([P, I64, I64, P, P, P, P, P], I),
@@ -196,8 +197,9 @@ def kq_selftest_div(a, b, mismatches, stream=None) -> None:
     _ok(lib().kq_selftest_div(_ptr(a), _ptr(b), a.numel(), _ptr(mismatches), _stream(stream)), "kq_selftest_div")
 
 
-def kq_accum_factor(A, H, accumulate: bool = False, trace=None, info=None, stream=None) -> None:
-    """H (+)= A^T A; A [T, d] bf16 (row stride may exceed d), H [d, d] fp32."""
+def kq_accum_factor(A, H, accumulate: bool = False, trace=None, info=None, stream=None, beside: bool = False) -> None:
+    """H (+)= A^T A; A [T, d] bf16 (row stride may exceed d), H [d, d] fp32. beside: this factor
+    runs beside other work, which gets the SMs that its last wave of tiles does not need."""
     if A.dim() != 2 or A.stride(1) != 1:
         raise ValueError("A must be 2-D with unit column stride")
     T, d = A.shape
@@ -205,8 +207,8 @@ def kq_accum_factor(A, H, accumulate: bool = False, trace=None, info=None, strea
     _need(H, "H", torch.float32, (d, d))
     _need(trace, "trace", torch.float64)
     _need(info, "info", torch.int32)
-    _ok(lib().kq_accum_factor(_ptr(A), T, d, A.stride(0), _ptr(H), int(accumulate), _ptr(trace),
-                              _ptr(info), _stream(stream)), "kq_accum_factor")
+    _ok(lib().kq_accum_factor_beside(_ptr(A), T, d, A.stride(0), _ptr(H), int(accumulate), _ptr(trace),
+                                     _ptr(info), int(beside), _stream(stream)), "kq_accum_factor")
 
 
 def kq_accum_drift_workspace(T: int, d: int) -> int:

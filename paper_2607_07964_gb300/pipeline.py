@@ -124,7 +124,7 @@ class LayerPipeline:
             ch += [(a, min(t1, a + q)) for a in range(t0, t1, q)]
         return ch
 
-    def _factor(self, which, A, H, trace, info, stream, ready=None) -> None:
+    def _factor(self, which, A, H, trace, info, stream, ready=None, beside: bool = False) -> None:
         """H = A^T A over the token chunks (Alg. 1 online statistic); `ready`, if given,
         holds one event per chunk that the stream waits on before using it."""
         ch = self._chunks(which, A.shape[0])
@@ -132,7 +132,7 @@ class LayerPipeline:
             if ready is not None:
                 stream.wait_event(ready[c])
             kq.kq_accum_factor(A if len(ch) == 1 else A[t0:t1], H, accumulate=c > 0, trace=trace if c == len(ch) - 1 else None,
-                               info=info, stream=stream)
+                               info=info, stream=stream, beside=beside)
 
     def _need_xt(self, Xt) -> None:
         if (self.alpha is None) != (Xt is None):
@@ -243,7 +243,7 @@ class LayerPipeline:
             kq.kq_accum_drift(Xt, X, self.D, info=self.info[2:3], ws=self.ws_drift, stream=s2)
             kq.kq_rotate_in(None, self.D, self.s_x, sign_v, kq.KQ_FWD, stream=s2)
             e_d.record(s2)
-        self._factor("G", G, self.HG, self.trace_g, self.info[2:3], s2, g_ready)
+        self._factor("G", G, self.HG, self.trace_g, self.info[2:3], s2, g_ready, beside=True)
         s2.wait_event(e_tx)                      # W (host path) and the X side of the traces
         kq.kq_compute_scales(W, None, self.HG, None, self.s_g, stream=s2)
         kq.kq_traces(None, None, self.HG, self.s_g, self.traces, stream=s2)
