@@ -890,7 +890,7 @@ def run_infer(args):
                                       f"q, k, v, o, gate, up, down in order on one stream",
                           "blocks": nb, "bits": bits, "tokens": B,
                           "l2": f"{wbytes / 1e9:.2f} GB of packed weights per step, larger than L2; no flush"},
-               "roofline": {"kernel": "kq_infer (infer_stream_kernel + infer_out_kernel) over all sublayers",
+               "roofline": {"kernel": "kq_infer (transform, infer_mma_kernel, transform) over all sublayers",
                             "bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm,
                             "traffic": None, "peak_source": f"{peak_src} HBM copy",
                             "bytes_per_step": wbytes},

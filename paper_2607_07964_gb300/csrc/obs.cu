@@ -102,7 +102,7 @@ __global__ void rowgrid_kernel(const float* __restrict__ W, int64_t d_out, int64
 // ~350-500 cycles for each of the seven hand-overs and ~5000 before the first column.
 // 4096 rows (128 CTAs): 30.3 k cycles, 14.6 us a block; the form with 8 lanes per row and a
 // shuffle per column took 25 us. With it the sweep of 1024 x 8192 went from 2.62 to 1.75 ms,
-// of 14336 x 4096 (three CTAs per SM) from 3.40 to 2.29 ms. A fully unrolled chain with one
+// of 14336 x 4096 (three CTAs per SM) from 3.40 to 2.29 ms (2.23 with the column sums' loads ahead). A fully unrolled chain with one
 // register per column and range tests that branch took 270 cycles a column; packed pairs
 // (f32x2 fma) for the updates, 16 against 30 instructions, took 170 to 145.
 constexpr int CW = 16;                      // columns per warp
