@@ -600,14 +600,23 @@ inline bool infer_mma_plan(int64_t d_out, int64_t d_in, int nc, MmaPlan* p) {
     return p->smem <= kInferSmemMax;
 }
 
+inline int mma_nc(int64_t B) { return B <= 2 ? 1 : B <= 5 ? 2 : 3; }   // column tiles of 8 for 3 B terms
+
+// Tokens of one product: all of them, or half where the terms of six to eight tokens do not fit
+// (d_in = 32768: 257 KB for a CTA's eighth of the groups, 182 KB for three or four tokens); 0 if
+// no product takes this size.
+inline int64_t mma_tokens(int64_t B, int64_t d_out, int64_t d_in) {
+    MmaPlan p;
+    if (infer_mma_plan(d_out, d_in, mma_nc(B), &p)) return B;
+    const int64_t h = cdiv(B, 2);
+    return infer_mma_plan(d_out, d_in, mma_nc(h), &p) ? h : 0;
+}
+
 template <int PB, int NC>
 kq_status launch_mma_nc(int64_t B, cudaStream_t st, const uint32_t* packed, const float* scale, const int32_t* zero,
                         int64_t d_out, int64_t d_in, int ng, int mid, const float* x, float* yp) {
     MmaPlan p;
-    if (!infer_mma_plan(d_out, d_in, NC, &p)) {
-        set_error("kq_infer: d_in=%lld is too large", (long long)d_in);
-        return KQ_ERR_UNSUPPORTED;
-    }
+    infer_mma_plan(d_out, d_in, NC, &p);   // fits: see mma_tokens
     static std::atomic<uint64_t> attr{0};
     KQ_TRY(once_per_device(attr, [&]() -> kq_status {
         KQ_CUDA(cudaFuncSetAttribute(infer_mma_kernel<PB, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -624,9 +633,11 @@ kq_status launch_mma_nc(int64_t B, cudaStream_t st, const uint32_t* packed, cons
 template <int PB>
 kq_status launch_mma(int64_t B, cudaStream_t st, const uint32_t* packed, const float* scale, const int32_t* zero,
                      int64_t d_out, int64_t d_in, int ng, int mid, const float* x, float* yp) {
-    if (B <= 2) return launch_mma_nc<PB, 1>(B, st, packed, scale, zero, d_out, d_in, ng, mid, x, yp);
-    if (B <= 5) return launch_mma_nc<PB, 2>(B, st, packed, scale, zero, d_out, d_in, ng, mid, x, yp);
-    return launch_mma_nc<PB, 3>(B, st, packed, scale, zero, d_out, d_in, ng, mid, x, yp);
+    switch (mma_nc(B)) {
+        case 1: return launch_mma_nc<PB, 1>(B, st, packed, scale, zero, d_out, d_in, ng, mid, x, yp);
+        case 2: return launch_mma_nc<PB, 2>(B, st, packed, scale, zero, d_out, d_in, ng, mid, x, yp);
+        default: return launch_mma_nc<PB, 3>(B, st, packed, scale, zero, d_out, d_in, ng, mid, x, yp);
+    }
 }
 
 // The sizes this call takes: d_in a rotation size of the library (2^k up to 2^15, 28 * 2^k up to
@@ -732,17 +743,21 @@ extern "C" kq_status kq_infer(const uint32_t* packed, const float* scale, const 
     }
     const int ng = group ? static_cast<int>(d_in / group) : 1;
     const int di = static_cast<int>(d_in), dn = static_cast<int>(d_out);
-    if (!sizes_ok(B, d_out, d_in, pb, ng, scale, zero)) {
+    const int64_t per = mma_tokens(B, d_out, d_in);
+    if (!sizes_ok(B, d_out, d_in, pb, ng, scale, zero) || per == 0) {
         set_error("kq_infer: d_in=%lld or d_out=%lld is beyond the rotation sizes", (long long)d_in, (long long)d_out);
         return KQ_ERR_UNSUPPORTED;
     }
     (void)info;   // no kernel of this call waits on a copy
     KQ_TRY(launch_rht<true>(B, stream, x, di, lgi, h28i, s_x, sign_v, xt));
     const int mid = 1 << (bits - 1);
-    kq_status st;
-    if (pb == 2) st = launch_mma<2>(B, stream, packed, scale, zero, d_out, d_in, ng, mid, xt, yp);
-    else if (pb == 4) st = launch_mma<4>(B, stream, packed, scale, zero, d_out, d_in, ng, mid, xt, yp);
-    else st = launch_mma<8>(B, stream, packed, scale, zero, d_out, d_in, ng, mid, xt, yp);
-    if (st != KQ_OK) return st;
+    for (int64_t t0 = 0; t0 < B; t0 += per) {
+        const int64_t n = std::min(per, B - t0);
+        const float* xn = xt + t0 * d_in;
+        float* yn = yp + t0 * d_out;
+        if (pb == 2) KQ_TRY(launch_mma<2>(n, stream, packed, scale, zero, d_out, d_in, ng, mid, xn, yn));
+        else if (pb == 4) KQ_TRY(launch_mma<4>(n, stream, packed, scale, zero, d_out, d_in, ng, mid, xn, yn));
+        else KQ_TRY(launch_mma<8>(n, stream, packed, scale, zero, d_out, d_in, ng, mid, xn, yn));
+    }
     return launch_rht<false>(B, stream, yp, dn, lgo, h28o, s_g, sign_u, y);
 }
