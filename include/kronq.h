@@ -149,9 +149,9 @@ KQ_API kq_status kq_selftest_div(const float* a, const float* b, int64_t n, unsi
 KQ_API kq_status kq_accum_factor(const uint16_t* A, int64_t T, int64_t d, int64_t lda, float* H,
                           int accumulate, double* trace, int* info, kq_stream_t stream);
 /* kq_accum_factor_beside: the same; with beside != 0 for a factor that runs beside other work, on
- *   a stream of lower priority: its tiles are launched a wave at a time, equally many each, so
- *   that the SMs which the last wave would leave idle are free for that work all the time. The
- *   same bits. */
+ *   a stream of lower priority: where that frees SMs (a ragged last wave, few waves), its tiles are
+ *   launched a wave at a time, equally many each, so that the SMs which the last wave would leave
+ *   idle are free for that work all the time. The same bits. */
 KQ_API kq_status kq_accum_factor_beside(const uint16_t* A, int64_t T, int64_t d, int64_t lda, float* H,
                                         int accumulate, double* trace, int* info, int beside,
                                         kq_stream_t stream);

@@ -646,11 +646,16 @@ extern "C" kq_status kq_accum_factor_beside(const uint16_t* A, int64_t T, int64_
         const int ks = ks_of(tiles, cdiv(T, KQ_SYRK_CHUNK_TOKENS));
         // Beside other work: a launch per wave, of equally many tiles, so that the SMs the last wave
         // would leave idle are free all the time (272 tiles on 152 SMs: twice 136; the inverse
-        // Cholesky's chain beside them does not wait a tile's whole sum for an SM). Layers, us:
-        // 4096 x 4096 and 131072 tokens 5743 -> 5528, 7168 x 4096 and 65536 6396 -> 6095; 16384 tokens
-        // 3419 -> 3432 (a tile takes 0.1 ms there) and 262144 8298 -> 8423 (a wave's tiles end up to
-        // 0.1 ms apart), hence the range. Fewer tiles at a time (91, three waves) 5676, 68 6438.
-        const int64_t waves = beside && ks == 1 && T >= 32768 && T < 196608 ? cdiv(tiles, num_sms()) : 1;
+        // Cholesky's chain beside them does not wait a tile's whole sum for an SM). Layers, us, one
+        // launch and waves: 4096 x 4096 and 131072 tokens 5865 -> 5560 (twice 136), 3584 x 4096 5406 ->
+        // 5005 (twice 105), 7168 x 4096 and 65536 6401 -> 5872 (six of 136). Only where 16 SMs or more
+        // come free, in up to six waves: each wave's tiles end up to 0.1 ms apart, and 8192 x 4096 (seven
+        // of 151, 65536 tokens) took 7128 -> 7199, 14336 x 4096 (21 of 152, 131072) 24103 -> 24723. 4096 x
+        // 4096 with 16384 tokens 3419 -> 3432 (a tile takes 0.1 ms there) and with 262144 in one call
+        // 8298 -> 8423, hence the range of T.
+        const bool by_wave = beside && ks == 1 && T >= 32768 && T < 196608;
+        const int64_t full = cdiv(tiles, num_sms());
+        const int64_t waves = by_wave && full <= 6 && num_sms() - cdiv(tiles, full) >= 16 ? full : 1;
         const int64_t per = cdiv(tiles, waves);   // tiles per launch
         auto go = [&](auto* kern) -> kq_status {
             for (int64_t t0 = 0; t0 < tiles; t0 += per) {
