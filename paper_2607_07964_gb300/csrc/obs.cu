@@ -506,6 +506,10 @@ __global__ void __launch_bounds__(OBS_THREADS, PER_SM) obs_block_kernel(
         g.scale = live ? gscale[r] : 1.0f;
         g.zero = live ? gzero[r] : 0.0f;
     }
+    if (!(fabsf(g.zero) <= 3.402823466e38f)) {   // scale underflowed to 0, or infinite: codes 0, E NaN
+        g.scale = __int_as_float(0x7FFFFFFF);
+        g.zero = 0.0f;
+    }
     g.ys = div_recip(g.scale);
     g.lo = __fsub_rn(0.0f, g.zero);
     g.hi = __fsub_rn(maxq, g.zero);
