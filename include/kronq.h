@@ -367,7 +367,9 @@ KQ_API kq_status kq_gptaq_p(const float* Dp, const float* Lt, int64_t n, float a
  *     Needs d_in % 4 == 0 and a 16-byte aligned W.
  *   Requirements: 1 <= bits <= 8, block == 128, group in {0, block}; with P also
  *   d_in % 16 == 0 and W, codes, Pt 16-byte aligned.
- *   info (nullable, device int): -KQ_ERR_TIMEOUT if a tensor-core pipeline wait gave up;
+ *   info (nullable, device int): -KQ_ERR_TIMEOUT if a bounded wait gave up: in either mode one of
+ *   the column loop (the codes of those columns are then not written, and col_loss and every
+ *   later column of those rows are NaN), in KQ_TRAIL_3XTF32 also one of the trailing update's pipeline;
  *   -KQ_ERR_NONFINITE if a value about to be quantized was NaN or infinite (a non-finite W',
  *   for example from a NaN weight; that row's codes and grids are then meaningless).
  *   ws: kq_obs_quantize_workspace(d_out, d_in, block, mode, with_p) bytes (with_p = 1 when

@@ -349,6 +349,23 @@ __device__ __forceinline__ void column_step(float w, const RowGrid& g, float2 d,
     }
 }
 
+// A thread whose wait ran out: NaN in its part of what the later updates read, so that even without a
+// word in info the columns after these and col_loss are NaN, not sums of what the workspace held.
+// (Places from the special registers again: nothing is kept in registers for this.)
+__device__ __forceinline__ void give_up(float* E, float* Eh, float* El, int64_t d_out, int64_t d_in, int64_t i0, int* info) {
+    uint32_t tid, cta;
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
+    asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(cta));
+    record_error(info, -KQ_ERR_TIMEOUT);
+    const int64_t r = static_cast<int64_t>(cta) * OBS_ROWS + (tid & 31), c0 = i0 + CW * (tid >> 5);
+    if (r >= d_out) return;
+#pragma unroll 1
+    for (int64_t c = c0; c < min(c0 + CW, d_in); ++c) {
+        E[r * d_in + c] = __int_as_float(0x7FFFFFFF);
+        if (Eh) Eh[r * d_in + c] = El[r * d_in + c] = __int_as_float(0x7FFFFFFF);
+    }
+}
+
 // VEC: d_in % 16 == 0 and W, codes (and pre_q) 16-byte aligned, so a lane's columns of W, E
 // and codes move as 16-byte vectors. HASP: with the GPTAQ correction; Pp is P's
 // diagonal block packed like R's, and the block's -Wpre goes to Q (fp32 trailing update)
@@ -522,7 +539,7 @@ __global__ void __launch_bounds__(OBS_THREADS, PER_SM) obs_block_kernel(
 #pragma unroll 1
         for (int p = 0; p < CW / PUB; ++p) {
             if (!mbar_wait(&pub[o * (CW / PUB) + p], 0, &abort_flag)) {
-                if (lane == 0) record_error(info, -KQ_ERR_TIMEOUT);
+                give_up(E, Eh, El, d_out, d_in, i0, info);
                 return;
             }
 #pragma unroll
