@@ -448,8 +448,10 @@ __device__ __forceinline__ float ratio_pow(float h, double a, float e) {
 }
 
 // a_j = ||W[:, j]||^2 and s_x[j] = (H_X[j][j] / a_j)^e (e = 1/4: Eq. rescale). Block (CS_X, CS_Y).
-__global__ void colscale_kernel(const float* __restrict__ W, int64_t d_out, int64_t d_in,
-                                const float* __restrict__ HX, int64_t hstride, float* __restrict__ s_x, float e) {
+template <int PER_SM>
+__global__ void __launch_bounds__(CS_X * CS_Y, PER_SM) colscale_kernel(const float* __restrict__ W, int64_t d_out, int64_t d_in,
+                                                                        const float* __restrict__ HX, int64_t hstride,
+                                                                        float* __restrict__ s_x, float e) {
     const int64_t j = static_cast<int64_t>(blockIdx.x) * CS_X + threadIdx.x;
     const double a = col_sumsq(W, d_out, d_in, j);
     if (threadIdx.y == 0 && j < d_in) s_x[j] = ratio_pow(HX[j * hstride], a, e);
@@ -465,7 +467,9 @@ __global__ void rowscale_kernel(const float* __restrict__ W, int64_t d_out, int6
 }
 
 // Squared column norms (a) and squared row norms (r) of W in fp64, for the BiIP statistics.
-__global__ void colnorm2_kernel(const float* __restrict__ W, int64_t d_out, int64_t d_in, double* __restrict__ a) {
+template <int PER_SM>
+__global__ void __launch_bounds__(CS_X * CS_Y, PER_SM) colnorm2_kernel(const float* __restrict__ W, int64_t d_out, int64_t d_in,
+                                                                        double* __restrict__ a) {
     const int64_t j = static_cast<int64_t>(blockIdx.x) * CS_X + threadIdx.x;
     const double v = col_sumsq(W, d_out, d_in, j);
     if (threadIdx.y == 0 && j < d_in) a[j] = v;
@@ -925,8 +929,8 @@ kq_status scales_impl(const float* W, int64_t d_out, int64_t d_in, const float* 
         return KQ_ERR_INVALID_ARG;
     }
     if (s_x) {
-        colscale_kernel<<<static_cast<unsigned>(cdiv(d_in, CS_X)), dim3(CS_X, CS_Y), 0, stream>>>(W, d_out, d_in, hx, xs, s_x,
-                                                                                               ex);
+        auto* kern = cs_per_sm(d_in) == 2 ? colscale_kernel<2> : colscale_kernel<1>;
+        kern<<<static_cast<unsigned>(cdiv(d_in, CS_X)), dim3(CS_X, CS_Y), 0, stream>>>(W, d_out, d_in, hx, xs, s_x, ex);
         KQ_LAUNCH_CHECK("colscale_kernel");
     }
     if (s_g) {
@@ -990,7 +994,8 @@ extern "C" kq_status kq_biip_stats(const float* W, int64_t d_out, int64_t d_in, 
     }
     double* a = static_cast<double*>(ws);
     double* r = a + d_in;
-    colnorm2_kernel<<<static_cast<unsigned>(cdiv(d_in, CS_X)), dim3(CS_X, CS_Y), 0, stream>>>(W, d_out, d_in, a);
+    auto* norms = cs_per_sm(d_in) == 2 ? colnorm2_kernel<2> : colnorm2_kernel<1>;
+    norms<<<static_cast<unsigned>(cdiv(d_in, CS_X)), dim3(CS_X, CS_Y), 0, stream>>>(W, d_out, d_in, a);
     KQ_LAUNCH_CHECK("colnorm2_kernel");
     rownorm2_kernel<<<static_cast<unsigned>(cdiv(d_out, 8)), 256, 0, stream>>>(W, d_out, d_in, r);
     KQ_LAUNCH_CHECK("rownorm2_kernel");

@@ -744,8 +744,9 @@ __global__ void __launch_bounds__(G_THREADS, 2) trailing_kernel(float* __restric
 
 // col_loss[j] = sum over rows of E[r][j]^2 in a fixed order (fp32 runs, fp64 across them).
 // Block (CS_X, CS_Y).
-__global__ void colloss_kernel(const float* __restrict__ E, int64_t d_out, int64_t d_in,
-                               float* __restrict__ col_loss) {
+template <int PER_SM>
+__global__ void __launch_bounds__(CS_X * CS_Y, PER_SM) colloss_kernel(const float* __restrict__ E, int64_t d_out, int64_t d_in,
+                                                                      float* __restrict__ col_loss) {
     const int64_t j = static_cast<int64_t>(blockIdx.x) * CS_X + threadIdx.x;
     const double a = col_sumsq(E, d_out, d_in, j);
     if (threadIdx.y == 0 && j < d_in && KQ_IN_RANGE(j, d_in)) col_loss[j] = static_cast<float>(a);
@@ -1144,7 +1145,8 @@ extern "C" kq_status kq_obs_quantize(float* W, int64_t d_out, int64_t d_in, cons
     }
     if (forked) KQ_CUDA(cudaStreamWaitEvent(stream, side->ev[1], 0));
     if (col_loss) {
-        colloss_kernel<<<static_cast<unsigned>(cdiv(d_in, CS_X)), dim3(CS_X, CS_Y), 0, stream>>>(o.E, d_out, d_in, col_loss);
+        auto* kern = cs_per_sm(d_in) == 2 ? colloss_kernel<2> : colloss_kernel<1>;
+        kern<<<static_cast<unsigned>(cdiv(d_in, CS_X)), dim3(CS_X, CS_Y), 0, stream>>>(o.E, d_out, d_in, col_loss);
         KQ_LAUNCH_CHECK("colloss_kernel");
     }
     return KQ_OK;
