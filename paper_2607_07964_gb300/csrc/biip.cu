@@ -170,11 +170,13 @@ __global__ void __launch_bounds__((1 << LG) / 16) rht_rows_reg_kernel(float* __r
 // warps of the other groups keep loads in flight while one group waits on its chunk.
 // (Seven groups of four chunks each, with the next row prefetched into registers,
 // measured 14.6-14.8 against 13.3 ms for the rotation stage of the 70B down_proj layer.)
-// Each thread's pre-factors are formed once and held in registers over its rows, and a group
-// meets only itself between its phases (it alone uses its exchange buffer): 14336 rows of 14336
-// 529.5 -> 460 -> 443.7 us (3.7 TB/s read and written). At the 72 registers two CTAs can share
-// about 150 bytes of the factors spill; one CTA per SM without spills was the slower one.
-template <int LG, bool POST>
+// HOLD: each thread's pre-factors are formed once and held in registers over its rows (spilling
+// some 150 bytes at the 72 registers two CTAs can share; one CTA per SM without spills was the
+// slower one), worth it from the third row of a CTA on: 14336 rows of 14336 529.5 -> 460 -> 443.7
+// us with the barriers below (3.7 TB/s read and written), 2048 82.7 -> 74.4, but 400 18.6 -> 20.6 and
+// 256 14.5 -> 16.5; with no row to hold them for, 256 rows take 13.0. A group meets only itself
+// between its phases (it alone uses its exchange buffer).
+template <int LG, bool POST, bool HOLD>
 __global__ void __launch_bounds__(14 * (1 << LG) / 16, LG == 9 ? 2 : 1) rht_rows28_reg_kernel(float* __restrict__ M, int64_t rows,
                                                                               int pre_mode, int post_mode,
                                                                               const int8_t* __restrict__ sign,
@@ -188,9 +190,11 @@ __global__ void __launch_bounds__(14 * (1 << LG) / 16, LG == 9 ? 2 : 1) rht_rows
     const int t = threadIdx.x, g = t / TG, tl = t - g * TG;
     float* buf = sm28 + N + g * P;                           // this group's exchange buffer
     const int tw = deposit_bits<(P - 1) & ~ML>(tl);
-    float f[CPG][16];   // this thread's pre-factors, the same for every row
+    float f[HOLD ? CPG : 1][16];   // this thread's pre-factors (HOLD: the same for every row)
+    if constexpr (HOLD) {
 #pragma unroll
-    for (int c = 0; c < CPG; ++c) factors16(pre_mode, sign, s, (g + G * c) * P + 16 * tl, f[c]);
+        for (int c = 0; c < CPG; ++c) factors16(pre_mode, sign, s, (g + G * c) * P + 16 * tl, f[c]);
+    }
     for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
 #pragma unroll
         for (int c = 0; c < CPG; ++c) {
@@ -205,8 +209,9 @@ __global__ void __launch_bounds__(14 * (1 << LG) / 16, LG == 9 ? 2 : 1) rht_rows
                 x[4 * q + 2] = w4.z;
                 x[4 * q + 3] = w4.w;
             }
+            if constexpr (!HOLD) factors16(pre_mode, sign, s, a * P + 16 * tl, f[0]);
 #pragma unroll
-            for (int k = 0; k < 16; ++k) x[k] *= f[c][k];
+            for (int k = 0; k < 16; ++k) x[k] *= f[HOLD ? c : 0][k];
             fwht_kbits<0xFu>(x);
             rr_transpose<LG, 1, true, true>(x, buf, tl, true, g);
             rr_transpose<LG, 2, true, true>(x, buf, tl, true, g);
@@ -246,8 +251,8 @@ __device__ __forceinline__ void fwht_regs(float (&x)[V]) {
 }
 
 // ------------------------------------------- row transform, n = 28 * 2^LG, LG in [4, 8]
-// 448 to 7168. A CTA takes 512 / P rows at a time (14336 values in shared memory, 56 KB, beside
-// a table of the pre-factors): a thread's 16 contiguous values take the first four stages in
+// 448 to 7168. A CTA takes up to 512 / P rows at a time (14336 values in shared memory, 56 KB, beside
+// a table of the factors): a thread's 16 contiguous values take the first four stages in
 // registers, the remaining LG - 4 stages (stride 16 in a chunk) one radix-2^(LG-4) pass through
 // shared memory, and then each of the 256 threads mixes two columns of a row (packed pairs) with
 // the dense +-1 sums of mix28 and writes 8-byte results. The stages, sums and factors are
@@ -255,24 +260,27 @@ __device__ __forceinline__ void fwht_regs(float (&x)[V]) {
 // additions a value of the mix (FP32 pipe) and HBM, which are close. rht_rows_kernel gave one
 // row to 256 threads, of which P mixed, and formed every factor again for every row: 8192 rows
 // of 896 146.7 -> 23.3 us, of 7168 359.5 -> 137.5 (3.4 TB/s read and written).
+// Few rows are spread over two CTAs per SM, fewer a CTA (64 rows of 896 10.4 -> 6.2 us; 8.3 with the
+// general kernel). A call has pre- or post-factors, never both, so the table holds either:
+// 1024 rows of 7168 with post-factors 45.3 -> 22.7 us (each thread had formed its 56 for each tile).
 // Quads of the shared copy are permuted within 128 bytes so that the 16-byte stores of 16
 // contiguous values per thread, and the later row accesses, hit distinct banks.
 __device__ __forceinline__ int quad_swz(int j) { return j ^ (((j >> 5) & 3) << 2); }
 
 template <int LG, bool POST>
-__global__ void __launch_bounds__(256, 2) rht_rows28_mid_kernel(float* __restrict__ M, int64_t rows, int pre_mode,
+__global__ void __launch_bounds__(256, 2) rht_rows28_mid_kernel(float* __restrict__ M, int64_t rows, int rows_per, int pre_mode,
                                                                 int post_mode, const int8_t* __restrict__ sign,
                                                                 const float* __restrict__ s, float inv_sqrt_n) {
     constexpr int P = 1 << LG, N = 28 * P, RPB = 512 / P, TILE = N * RPB;   // 14336
     constexpr int R = 1 << (LG - 4);   // radix of the second pass
     extern __shared__ __align__(16) float smid[];
     float* v = smid;             // [RPB][N]
-    float* pf = smid + TILE;     // [N] pre-factors
-    for (int j = threadIdx.x; j < N; j += 256) pf[j] = factor(pre_mode, sign, s, j);
-    const int64_t tiles = (rows + RPB - 1) / RPB;
+    float* pf = smid + TILE;     // [N] pre-factors (POST: post-factors over sqrt(n))
+    for (int j = threadIdx.x; j < N; j += 256) pf[j] = POST ? factor(post_mode, sign, s, j) * inv_sqrt_n : factor(pre_mode, sign, s, j);
+    const int64_t tiles = (rows + rows_per - 1) / rows_per;
     for (int64_t w = blockIdx.x; w < tiles; w += gridDim.x) {
-        float* base = M + w * TILE;
-        const int live = static_cast<int>(min(static_cast<int64_t>(RPB), rows - w * RPB)) * N;   // values of this tile
+        float* base = M + w * rows_per * N;
+        const int live = static_cast<int>(min(static_cast<int64_t>(rows_per), rows - w * rows_per)) * N;   // values of this tile
         __syncthreads();   // the previous tile's columns have been read (and pf is there)
 #pragma unroll 2
         for (int e = 16 * threadIdx.x; e < TILE; e += 16 * 256) {
@@ -282,7 +290,7 @@ __global__ void __launch_bounds__(256, 2) rht_rows28_mid_kernel(float* __restric
             const float4* pq = reinterpret_cast<const float4*>(pf + (RPB == 1 ? e : e % N));
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const float4 a = src[q], f = pq[q];
+                const float4 a = src[q], f = POST ? make_float4(1.0f, 1.0f, 1.0f, 1.0f) : pq[q];
                 x[4 * q] = __fmul_rn(a.x, f.x);
                 x[4 * q + 1] = __fmul_rn(a.y, f.y);
                 x[4 * q + 2] = __fmul_rn(a.z, f.z);
@@ -315,11 +323,9 @@ __global__ void __launch_bounds__(256, 2) rht_rows28_mid_kernel(float* __restric
                 for (int a = 0; a < 28; ++a) x[a] = *reinterpret_cast<const float2*>(v + quad_swz(row * N + a * P + b));
                 float* dst = base + row * N + b;
                 mix28_pairs(x, [&](int a, float2 y) {
-                    const int j = a * P + b;
-                    const float f0 = POST ? factor(post_mode, sign, s, j) * inv_sqrt_n : inv_sqrt_n;
-                    const float f1 = POST ? factor(post_mode, sign, s, j + 1) * inv_sqrt_n : inv_sqrt_n;
+                    const float2 f = POST ? *reinterpret_cast<const float2*>(pf + a * P + b) : make_float2(inv_sqrt_n, inv_sqrt_n);
                     if (KQ_IN_RANGE((dst - M) + a * P + 1, rows * N))
-                        *reinterpret_cast<float2*>(dst + a * P) = make_float2(y.x * f0, y.y * f1);
+                        *reinterpret_cast<float2*>(dst + a * P) = make_float2(y.x * f.x, y.y * f.y);
                 });
             }
         }
@@ -738,19 +744,18 @@ kq_status launch_rows28_reg(float* M, int64_t rows, int pre, int post, const int
     constexpr size_t smem = (28 * static_cast<size_t>(P) + 14 * static_cast<size_t>(P)) * sizeof(float);
     static std::atomic<uint64_t> attr{0};
     KQ_TRY(once_per_device(attr, [&]() -> kq_status {
-        KQ_CUDA(cudaFuncSetAttribute(rht_rows28_reg_kernel<LG, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(smem)));
-        KQ_CUDA(cudaFuncSetAttribute(rht_rows28_reg_kernel<LG, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(smem)));
+        for (auto* kern : {rht_rows28_reg_kernel<LG, true, false>, rht_rows28_reg_kernel<LG, false, true>,
+                           rht_rows28_reg_kernel<LG, false, false>})
+            KQ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
         return KQ_OK;
     }));
     const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(static_cast<int64_t>((227 * 1024) / smem), 2048 / T));
     const int64_t grid = std::min<int64_t>(rows, static_cast<int64_t>(num_sms()) * per_sm);
     const float isn = static_cast<float>(1.0 / sqrt(static_cast<double>(28 * P)));
-    if (post == F_NONE)
-        rht_rows28_reg_kernel<LG, false><<<static_cast<unsigned>(grid), T, smem, stream>>>(M, rows, pre, post, sign, s, isn);
-    else
-        rht_rows28_reg_kernel<LG, true><<<static_cast<unsigned>(grid), T, smem, stream>>>(M, rows, pre, post, sign, s, isn);
+    // pre-factors (the forms with post-factors have none) held over a CTA's rows from the third one on
+    auto* kern = post != F_NONE ? rht_rows28_reg_kernel<LG, true, false>
+                 : rows > 2 * grid ? rht_rows28_reg_kernel<LG, false, true> : rht_rows28_reg_kernel<LG, false, false>;
+    kern<<<static_cast<unsigned>(grid), T, smem, stream>>>(M, rows, pre, post, sign, s, isn);
     KQ_LAUNCH_CHECK("rht_rows28_reg_kernel");
     return KQ_OK;
 }
@@ -768,12 +773,12 @@ kq_status launch_rows28_mid(float* M, int64_t rows, int pre, int post, const int
                                      static_cast<int>(smem)));
         return KQ_OK;
     }));
-    const int64_t grid = std::min<int64_t>(cdiv(rows, RPB), static_cast<int64_t>(num_sms()) * 2);
+    const int64_t slots = static_cast<int64_t>(num_sms()) * 2;
+    const int per = static_cast<int>(std::min<int64_t>(RPB, cdiv(rows, slots)));   // few rows: spread over the CTAs
+    const unsigned grid = static_cast<unsigned>(std::min<int64_t>(cdiv(rows, per), slots));
     const float isn = static_cast<float>(1.0 / sqrt(static_cast<double>(N)));
-    if (post == F_NONE)
-        rht_rows28_mid_kernel<LG, false><<<static_cast<unsigned>(grid), 256, smem, stream>>>(M, rows, pre, post, sign, s, isn);
-    else
-        rht_rows28_mid_kernel<LG, true><<<static_cast<unsigned>(grid), 256, smem, stream>>>(M, rows, pre, post, sign, s, isn);
+    auto* kern = post == F_NONE ? rht_rows28_mid_kernel<LG, false> : rht_rows28_mid_kernel<LG, true>;
+    kern<<<grid, 256, smem, stream>>>(M, rows, per, pre, post, sign, s, isn);
     KQ_LAUNCH_CHECK("rht_rows28_mid_kernel");
     return KQ_OK;
 }
@@ -1087,7 +1092,6 @@ extern "C" kq_status kq_rotate_out(float* W, int64_t d_out, int64_t d_in, float*
 
 // Used by the check-only revert (check.cu).
 namespace kq {
-// Used by the check-only revert (check.cu).
 kq_status rotate_rows_inv(float* M, int64_t rows, int64_t n, const float* s, const int8_t* sign,
                           cudaStream_t stream) {
     return rows_transform(M, rows, n, F_NONE, s ? F_SDIV : F_SIGN, sign, s, stream);
