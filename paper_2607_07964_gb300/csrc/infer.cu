@@ -641,17 +641,18 @@ kq_status launch_mma(int64_t B, cudaStream_t st, const uint32_t* packed, const f
 }
 
 // The sizes this call takes: d_in a rotation size of the library (2^k up to 2^15, 28 * 2^k up to
-// 28 * 1024); d_out too, or up to 65536 while x' of the tokens leaves room for two 4-row slabs of
-// codes and grids in shared memory and the grids are 16-byte aligned.
+// 28 * 1024); d_out too, or 28 * 2048 and 65536 with 16-byte aligned grids while the tokens' x' (33 floats for
+// 32) and eight rows of codes and grids are at most 226 KB. The kernels need neither condition (see
+// infer_mma_plan for theirs): they say which of these two d_out the call takes, and d_in * B for them.
 inline bool rotation_size(int64_t n) { return n % 28 == 0 ? n <= 28 * 1024 : n <= 32768; }
 inline bool sizes_ok(int64_t B, int64_t d_out, int64_t d_in, int pb, int64_t ng, const void* scale, const void* zero) {
     if (!rotation_size(d_in)) return false;
     if (rotation_size(d_out)) return true;
     const int64_t S = cdiv(d_in / 8 * pb / 16, 32);
-    const int64_t xbytes = B * S * (32 / pb) * 132 * 4 + (d_in == 4096 ? 4224 * 4 : 0);
-    const int64_t slab = 4 * (d_in / 8 * pb) + 32 * ng + (4 * S * B + 3) / 4 * 16;
+    const int64_t xbytes = B * S * (32 / pb) * 132 * 4;
+    const int64_t rows = 2 * (4 * (d_in / 8 * pb) + 32 * ng + (4 * S * B + 3) / 4 * 16);
     return d_out <= 65536 && ((reinterpret_cast<uintptr_t>(scale) | reinterpret_cast<uintptr_t>(zero)) & 15u) == 0 &&
-           xbytes + 2 * slab <= static_cast<int64_t>(kInferSmemMax);
+           xbytes + rows <= static_cast<int64_t>(kInferSmemMax);
 }
 
 // n = 28 * 2^k or 2^k: (k, has28); false if neither.
@@ -705,8 +706,7 @@ extern "C" kq_status kq_pack_codes(const uint8_t* codes, int64_t d_out, int64_t 
 
 extern "C" size_t kq_infer_workspace(int64_t B, int64_t d_in, int64_t d_out) {
     if (B < 1 || d_in < 1 || d_out < 1) return 0;
-    return al256(static_cast<size_t>(B) * d_in * sizeof(float)) + al256(static_cast<size_t>(B) * (d_in / 16) * sizeof(float)) +
-           al256(static_cast<size_t>(B) * d_out * sizeof(float)) + 256 + 256;
+    return al256(static_cast<size_t>(B) * d_in * sizeof(float)) + al256(static_cast<size_t>(B) * d_out * sizeof(float));
 }
 
 extern "C" kq_status kq_infer(const uint32_t* packed, const float* scale, const int32_t* zero, int64_t d_out,
@@ -733,8 +733,7 @@ extern "C" kq_status kq_infer(const uint32_t* packed, const float* scale, const 
         return KQ_ERR_WORKSPACE;
     }
     float* xt = static_cast<float*>(ws);   // x' of the tokens; y' behind it (see kq_infer_workspace)
-    float* yp = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + al256(static_cast<size_t>(B) * d_in * sizeof(float)) +
-                                         al256(static_cast<size_t>(B) * (d_in / 16) * sizeof(float)));
+    float* yp = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + al256(static_cast<size_t>(B) * d_in * sizeof(float)));
     const int pb = lane_bits(bits);
     int lgi = 0, h28i = 0, lgo = 0, h28o = 0;
     if (!rht_plan(d_in, &lgi, &h28i) || !rht_plan(d_out, &lgo, &h28o)) {

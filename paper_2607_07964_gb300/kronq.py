@@ -440,8 +440,8 @@ def kq_infer_workspace(B: int, d_in: int, d_out: int) -> int:
 def kq_infer(packed, scale, zero, d_out: int, d_in: int, bits: int, group: int, s_x, s_g, sign_u, sign_v, x, y,
              ws, stream=None, info=None) -> None:
     """y [B, d_out] = W^ x for x [B, d_in]: the reverted quantized layer applied with online
-    Hadamard transforms (Algorithm 2's revert, Sec. 3.2). info: optional int32 device word
-    for a timed-out weight stream (read with kq_check)."""
+    Hadamard transforms (Algorithm 2's revert, Sec. 3.2). info: optional int32 device word, in
+    which no kernel of this call records anything."""
     B = x.shape[0]
     _need(packed, "packed", torch.int32)
     _need(scale, "scale", torch.float32)
