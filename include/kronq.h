@@ -401,7 +401,8 @@ KQ_API kq_status kq_obs_quantize(float* W, int64_t d_out, int64_t d_in, const fl
  *   for group 128), s_x [d_in], s_g [d_out] and the RHT signs of the quantization.
  *   fp32 throughout: the codes less the middle code are exact in bf16 and x' is the exact sum of
  *   three bf16 terms, so the tensor cores' products are exact and summed in fp32 (per group
- *   scale (sum (q - c) x' - (zero - c) sum x')).
+ *   scale (sum (q - c) x' - (zero - c) sum x')). The tensor cores do not round each of these
+ *   additions to nearest as a chain of fp32 additions does (16 products at a time).
  *   ws: kq_infer_workspace(B, d_in, d_out) bytes, 256-byte aligned. packed, x, y, s_x, s_g
  *   16-byte aligned, the signs 4-byte aligned, d_out % 4 == 0; s_x, s_g required (not NULL). d_in and d_out need Hadamard constructions (2^k or 28 * 2^k).
  *   info: optional device error word (see kq_check); no kernel of this call records in it.

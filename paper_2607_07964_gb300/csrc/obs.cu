@@ -366,7 +366,7 @@ __device__ __forceinline__ void give_up(float* E, float* Eh, float* El, int64_t 
     }
 }
 
-// VEC: d_in % 16 == 0 and W, codes (and pre_q) 16-byte aligned, so a lane's columns of W, E
+// VEC: d_in % 16 == 0 and W and codes 16-byte aligned, so a lane's columns of W, E
 // and codes move as 16-byte vectors. HASP: with the GPTAQ correction; Pp is P's
 // diagonal block packed like R's, and the block's -Wpre goes to Q (fp32 trailing update)
 // or to Qh + Ql (tensor-core trailing update). FUSE: the previous block's update of this

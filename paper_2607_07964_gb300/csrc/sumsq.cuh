@@ -19,7 +19,9 @@ namespace kq {
 // Registers (80 a thread: one CTA per SM; 64: two): one while every CTA has an SM of its own, 4096
 // x 4096 18.8 us against 22.3 and 8192 x 1024 26.7 against 35.0; two beyond, where the second
 // CTA fills the SM: 1024 x 8192 14.8 -> 12.4, 256 x 28672 22.6 -> 14.4 (18.5 without loads ahead,
-// 56 registers), 8192 x 28672 187 -> 160 (197).
+// 56 registers), 8192 x 28672 187 -> 160 (197). Just past one CTA per SM it depends on the rows
+// (scales of both sides, one and two: 256 x 4896 16.5 and 14.4, 4096 x 4896 39.0 and 43.1, 4096 x
+// 7168 55.6 and 52.1, 14336 x 4896 154.9 and 148.6).
 constexpr int CS_X = 32, CS_Y = 16, CS_U = 16;
 
 inline int cs_per_sm(int64_t cols) { return cdiv(cols, CS_X) > num_sms() ? 2 : 1; }
