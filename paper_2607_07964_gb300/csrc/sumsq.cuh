@@ -16,7 +16,7 @@ namespace kq {
 // 112.6 -> 65.5 us with the loads ahead, 4096 x 4096 41.0 -> 26.6). A second thread row of loaders
 // for each chain, its sums handed over through shared memory, took 69.6 and 26.6 us, and 22.5
 // against 18.5 at 1024 x 8192.
-// Registers (80 a thread: one CTA per SM; 64: two): one while every CTA has an SM of its own, 4096
+// Registers (95 a thread: one CTA per SM; 64: two): one while every CTA has an SM of its own, 4096
 // x 4096 18.8 us against 22.3 and 8192 x 1024 26.7 against 35.0; two beyond, where the second
 // CTA fills the SM: 1024 x 8192 14.8 -> 12.4, 256 x 28672 22.6 -> 14.4 (18.5 without loads ahead,
 // 56 registers), 8192 x 28672 187 -> 160 (197). Just past one CTA per SM it depends on the rows
