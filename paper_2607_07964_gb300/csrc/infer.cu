@@ -593,8 +593,9 @@ inline bool infer_mma_plan(int64_t d_out, int64_t d_in, int nc, MmaPlan* p) {
         const int64_t part = IM_ROWS * 8 * nc;   // partial sums; their totals take at most as much
         return static_cast<size_t>(std::max(g * nc * IM_GW, part) + std::max(g * (8 * nc + 2 * IM_ROWS), part)) * 4;
     };
+    const int sms = num_sms();
     p->C = 1;
-    while (p->C < 8 && 2 * p->C <= G && (tiles * p->C < num_sms() || bytes(cdiv(G, p->C)) > 112 * 1024)) p->C *= 2;
+    while (p->C < 8 && 2 * p->C <= G && (tiles * p->C < sms || bytes(cdiv(G, p->C)) > 112 * 1024)) p->C *= 2;
     p->gmax = static_cast<int>(cdiv(G, p->C));
     p->smem = bytes(p->gmax);
     return p->smem <= kInferSmemMax;
@@ -602,21 +603,18 @@ inline bool infer_mma_plan(int64_t d_out, int64_t d_in, int nc, MmaPlan* p) {
 
 inline int mma_nc(int64_t B) { return B <= 2 ? 1 : B <= 5 ? 2 : 3; }   // column tiles of 8 for 3 B terms
 
-// Tokens of one product: all of them, or half where the terms of six to eight tokens do not fit
-// (d_in = 32768: 257 KB for a CTA's eighth of the groups, 182 KB for three or four tokens); 0 if
-// no product takes this size.
-inline int64_t mma_tokens(int64_t B, int64_t d_out, int64_t d_in) {
-    MmaPlan p;
-    if (infer_mma_plan(d_out, d_in, mma_nc(B), &p)) return B;
+// Tokens of one product and its plan: all of them, or half where the terms of six to eight tokens do
+// not fit (d_in = 32768: 257 KB for a CTA's eighth of the groups, 182 KB for three or four tokens, which
+// have one plan); 0 if no product takes this size.
+inline int64_t mma_tokens(int64_t B, int64_t d_out, int64_t d_in, MmaPlan* p) {
+    if (infer_mma_plan(d_out, d_in, mma_nc(B), p)) return B;
     const int64_t h = cdiv(B, 2);
-    return infer_mma_plan(d_out, d_in, mma_nc(h), &p) ? h : 0;
+    return infer_mma_plan(d_out, d_in, mma_nc(h), p) ? h : 0;
 }
 
 template <int PB, int NC>
-kq_status launch_mma_nc(int64_t B, cudaStream_t st, const uint32_t* packed, const float* scale, const int32_t* zero,
-                        int64_t d_out, int64_t d_in, int ng, int mid, const float* x, float* yp) {
-    MmaPlan p;
-    infer_mma_plan(d_out, d_in, NC, &p);   // fits: see mma_tokens
+kq_status launch_mma_nc(const MmaPlan& p, int64_t B, cudaStream_t st, const uint32_t* packed, const float* scale,
+                        const int32_t* zero, int64_t d_out, int64_t d_in, int ng, int mid, const float* x, float* yp) {
     static std::atomic<uint64_t> attr{0};
     KQ_TRY(once_per_device(attr, [&]() -> kq_status {
         KQ_CUDA(cudaFuncSetAttribute(infer_mma_kernel<PB, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -631,12 +629,12 @@ kq_status launch_mma_nc(int64_t B, cudaStream_t st, const uint32_t* packed, cons
     return KQ_OK;
 }
 template <int PB>
-kq_status launch_mma(int64_t B, cudaStream_t st, const uint32_t* packed, const float* scale, const int32_t* zero,
-                     int64_t d_out, int64_t d_in, int ng, int mid, const float* x, float* yp) {
+kq_status launch_mma(const MmaPlan& p, int64_t B, cudaStream_t st, const uint32_t* packed, const float* scale,
+                     const int32_t* zero, int64_t d_out, int64_t d_in, int ng, int mid, const float* x, float* yp) {
     switch (mma_nc(B)) {
-        case 1: return launch_mma_nc<PB, 1>(B, st, packed, scale, zero, d_out, d_in, ng, mid, x, yp);
-        case 2: return launch_mma_nc<PB, 2>(B, st, packed, scale, zero, d_out, d_in, ng, mid, x, yp);
-        default: return launch_mma_nc<PB, 3>(B, st, packed, scale, zero, d_out, d_in, ng, mid, x, yp);
+        case 1: return launch_mma_nc<PB, 1>(p, B, st, packed, scale, zero, d_out, d_in, ng, mid, x, yp);
+        case 2: return launch_mma_nc<PB, 2>(p, B, st, packed, scale, zero, d_out, d_in, ng, mid, x, yp);
+        default: return launch_mma_nc<PB, 3>(p, B, st, packed, scale, zero, d_out, d_in, ng, mid, x, yp);
     }
 }
 
@@ -742,7 +740,8 @@ extern "C" kq_status kq_infer(const uint32_t* packed, const float* scale, const 
     }
     const int ng = group ? static_cast<int>(d_in / group) : 1;
     const int di = static_cast<int>(d_in), dn = static_cast<int>(d_out);
-    const int64_t per = mma_tokens(B, d_out, d_in);
+    MmaPlan plan;
+    const int64_t per = mma_tokens(B, d_out, d_in, &plan);
     if (!sizes_ok(B, d_out, d_in, pb, ng, scale, zero) || per == 0) {
         set_error("kq_infer: d_in=%lld or d_out=%lld is beyond the rotation sizes", (long long)d_in, (long long)d_out);
         return KQ_ERR_UNSUPPORTED;
@@ -754,9 +753,9 @@ extern "C" kq_status kq_infer(const uint32_t* packed, const float* scale, const 
         const int64_t n = std::min(per, B - t0);
         const float* xn = xt + t0 * d_in;
         float* yn = yp + t0 * d_out;
-        if (pb == 2) KQ_TRY(launch_mma<2>(n, stream, packed, scale, zero, d_out, d_in, ng, mid, xn, yn));
-        else if (pb == 4) KQ_TRY(launch_mma<4>(n, stream, packed, scale, zero, d_out, d_in, ng, mid, xn, yn));
-        else KQ_TRY(launch_mma<8>(n, stream, packed, scale, zero, d_out, d_in, ng, mid, xn, yn));
+        if (pb == 2) KQ_TRY(launch_mma<2>(plan, n, stream, packed, scale, zero, d_out, d_in, ng, mid, xn, yn));
+        else if (pb == 4) KQ_TRY(launch_mma<4>(plan, n, stream, packed, scale, zero, d_out, d_in, ng, mid, xn, yn));
+        else KQ_TRY(launch_mma<8>(plan, n, stream, packed, scale, zero, d_out, d_in, ng, mid, xn, yn));
     }
     return launch_rht<false>(B, stream, yp, dn, lgo, h28o, s_g, sign_u, y);
 }
