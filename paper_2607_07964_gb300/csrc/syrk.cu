@@ -466,6 +466,7 @@ __device__ __forceinline__ void gram_tc_body(const CUtensorMap* a0, const CUtens
         __syncthreads();
     if (*abort_flag && threadIdx.x == 0) record_error(info, -KQ_ERR_TIMEOUT);
     if (warp == 1) {
+        __syncwarp();   // its lanes come from different roles, and the cluster's barrier is not a warp's
         tc_fence_after();
         tmem_dealloc(tmem, TMEM_COLS);
     }
